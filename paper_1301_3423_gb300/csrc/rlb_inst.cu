@@ -48,8 +48,7 @@ cudaError_t fields(const void* src, const StepParams& p, const FieldOut& f, doub
                    int block0, int block1, cudaStream_t s) {
   const int blocks = block1 - block0;
   if (blocks <= 0) return cudaSuccess;
-  // the modulo wrap only for lattices with a periodic axis shorter than the stencil reach
-  if (pull && p.general)
+  if (pull && p.has_wall)
     k_fields<L, S, true, true><<<blocks, kMomThreads, 0, s>>>((const T*)src, p, f, partial, status, block0);
   else if (pull)
     k_fields<L, S, true, false><<<blocks, kMomThreads, 0, s>>>((const T*)src, p, f, partial, status, block0);
@@ -105,34 +104,8 @@ extern const Launchers RLB_NAME(RLB_INST_ORDER, RLB_INST_STORAGE) = {
     step, fields, init, convert_pops, inst::kVariants, batch_step, batch_blocks_per_sm, pipe_step, pipe_batch_step};
 
 #if RLB_INST_ORDER == 3 && RLB_INST_STORAGE == 0
-// Second pass of the conserved-density sums: one block adds the per-block partials in a fixed
-// order (thread t takes blocks t, t + 256, ...; then a shuffle and shared-memory tree), so the
-// totals are bitwise reproducible.
-__global__ void __launch_bounds__(kReduceThreads) k_reduce_partials(const double* __restrict__ partial, int nblocks,
-                                                                     double* __restrict__ totals) {
-  __shared__ double ws[kReduceThreads / 32][5];
-  double d[5] = {0, 0, 0, 0, 0};
-  for (int b = threadIdx.x; b < nblocks; b += kReduceThreads)
-#pragma unroll
-    for (int k = 0; k < 5; ++k) d[k] += partial[(long long)b * 5 + k];
-#pragma unroll
-  for (int k = 0; k < 5; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d[k] += __shfl_down_sync(0xffffffffu, d[k], o);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < 5; ++k) ws[warp][k] = d[k];
-  __syncthreads();
-  if (threadIdx.x < 5) {
-    double s = 0.0;
-    for (int w = 0; w < kReduceThreads / 32; ++w) s += ws[w][threadIdx.x];
-    totals[threadIdx.x] = s;
-  }
-}
-
 cudaError_t launch_reduce_partials(const double* partial, int nblocks, double* totals, cudaStream_t s) {
-  k_reduce_partials<<<1, kReduceThreads, 0, s>>>(partial, nblocks, totals);
+  k_reduce_partials<<<5, kReduceThreads, 0, s>>>(partial, nblocks, totals);
   return cudaGetLastError();
 }
 #endif

@@ -213,6 +213,43 @@ __device__ __forceinline__ long long pull_index(const Cell& cl, const StepParams
 }
 
 
+// The in-plane index every pull of one cell needs, as one source offset per axis and velocity
+// component (at most 13 values an axis): a population's source is x[vx] + y[vy] + z[vz], two adds,
+// whatever the boundary.  Worked out once per cell (wrap, modulo wrap of an axis shorter than the
+// reach, or clamp), where pull_index tests and wraps three coordinates for each of the Q
+// populations: on a 1 x 1 x N tube, whose x and y take the modulo, that was most of a step.
+template <class L>
+struct PullTab {
+  int x[2 * L::VMAX_X + 1], y[2 * L::VMAX_Y + 1], z[2 * L::VMAX_Z + 1];
+
+  static __device__ __forceinline__ int wrap(int s, int n, int bc) {
+    if ((unsigned)s < (unsigned)n) return s;
+    if (bc) return s < 0 ? 0 : n - 1;
+    s += s < 0 ? n : -n;
+    if ((unsigned)s < (unsigned)n) return s;
+    s %= n;
+    return s < 0 ? s + n : s;
+  }
+  __device__ __forceinline__ PullTab(const Cell& cl, const StepParams& p) {
+#pragma unroll
+    for (int j = 0; j <= 2 * L::VMAX_X; ++j) x[j] = wrap(cl.x - (j - L::VMAX_X), p.nx, p.bc[0]);
+#pragma unroll
+    for (int j = 0; j <= 2 * L::VMAX_Y; ++j) y[j] = wrap(cl.y - (j - L::VMAX_Y), p.ny, p.bc[1]) * p.nx;
+#pragma unroll
+    for (int j = 0; j <= 2 * L::VMAX_Z; ++j) z[j] = wrap(cl.z - (j - L::VMAX_Z), p.nz, p.bc[2]) * p.nxy;
+  }
+  // index into the population buffer: plane offset of I (its mirror partner's beyond a wall) plus
+  // the in-plane index
+  template <int I, bool WALLS>
+  __device__ __forceinline__ long long index(const Cell& cl, const StepParams& p) const {
+    if constexpr (WALLS) {
+      if (beyond_wall<L, I>(cl, p)) return (long long)(I ^ 1) * p.cells + cl.c;
+    }
+    return (long long)I * p.cells +
+           (unsigned)(x[L::VX[I] + L::VMAX_X] + y[L::VY[I] + L::VMAX_Y] + z[L::VZ[I] + L::VMAX_Z]);
+  }
+};
+
 // Pull offset of population I from the cell's own index when only the x coordinate can leave the
 // lattice (rows whose y and z are interior): the constant offset with x wrapped or clamped, or the
 // cell's own reversed population beyond a bounce-back wall in x.
@@ -1076,7 +1113,8 @@ __global__ void __launch_bounds__(kStepThreads, StepShape<S, VARIANT>::kMinBlock
 // ---------------------------------------------------------------------------------------------
 // float-float arithmetic: a value as the unevaluated sum hi + lo of two floats (|lo| <= ulp(hi)/2),
 // built from the error-free transformations of Dekker and Knuth (two-sum; two-product by FMA).
-// About 44 bits of significand, at float-pipe speed.
+// About 44 bits of significand, at float-pipe speed: GB300 runs 64 float operations for each double
+// one, and a float-float operation takes 7 to 12 of them.
 // ---------------------------------------------------------------------------------------------
 struct FF {
   float hi, lo;
@@ -1086,56 +1124,89 @@ __device__ __forceinline__ FF ff_from(double x) {
   const float hi = (float)x;
   return FF{hi, (float)(x - (double)hi)};
 }
+__host__ __device__ constexpr FF ff_const(double x) { return FF{(float)x, (float)(x - (double)(float)x)}; }
+__device__ __forceinline__ double ff_double(FF a) { return (double)a.hi + (double)a.lo; }
 
 __device__ __forceinline__ FF ff_neg(FF a) { return FF{-a.hi, -a.lo}; }
 
 // hi + lo of a + b exactly (Knuth's two-sum)
 __device__ __forceinline__ FF two_sum(float a, float b) {
-  const float s = a + b;
-  const float bb = s - a;
-  return FF{s, (a - (s - bb)) + (b - bb)};
+  const float s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  return FF{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
 }
 
 __device__ __forceinline__ FF fast_two_sum(float a, float b) {  // |a| >= |b|
-  const float s = a + b;
-  return FF{s, b - (s - a)};
+  const float s = __fadd_rn(a, b);
+  return FF{s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+
+// hi + lo of a b exactly
+__device__ __forceinline__ FF two_prod(float a, float b) {
+  const float p = __fmul_rn(a, b);
+  return FF{p, fmaf(a, b, -p)};
 }
 
 __device__ __forceinline__ FF ff_add(FF a, FF b) {
   const FF s = two_sum(a.hi, b.hi);
   return fast_two_sum(s.hi, s.lo + (a.lo + b.lo));
 }
+__device__ __forceinline__ FF ff_add(FF a, float b) {
+  const FF s = two_sum(a.hi, b);
+  return fast_two_sum(s.hi, s.lo + a.lo);
+}
+__device__ __forceinline__ FF ff_sub(FF a, FF b) { return ff_add(a, ff_neg(b)); }
 
 __device__ __forceinline__ FF ff_mul(FF a, FF b) {
-  const float p = a.hi * b.hi;
-  const float e = fmaf(a.hi, b.hi, -p);  // exact error of the product
-  return fast_two_sum(p, e + fmaf(a.hi, b.lo, a.lo * b.hi));
+  const FF p = two_prod(a.hi, b.hi);
+  return fast_two_sum(p.hi, p.lo + fmaf(a.hi, b.lo, a.lo * b.hi));
+}
+__device__ __forceinline__ FF ff_mul(FF a, float b) {
+  const FF p = two_prod(a.hi, b);
+  return fast_two_sum(p.hi, fmaf(a.lo, b, p.lo));
+}
+// a times a power of two (exact)
+__device__ __forceinline__ FF ff_scale2(FF a, float k) { return FF{a.hi * k, a.lo * k}; }
+
+// acc + m u: the product's error and the sum's error both kept
+__device__ __forceinline__ FF ff_mac(FF acc, float m, float u) {
+  const FF p = two_prod(m, u);
+  const FF s = two_sum(acc.hi, p.hi);
+  return FF{s.hi, s.lo + (acc.lo + p.lo)};
+}
+__device__ __forceinline__ FF ff_mac(FF acc, FF m, FF u) {
+  const FF p = two_prod(m.hi, u.hi);
+  const FF s = two_sum(acc.hi, p.hi);
+  return FF{s.hi, s.lo + (acc.lo + fmaf(m.hi, u.lo, fmaf(m.lo, u.hi, p.lo)))};
+}
+__device__ __forceinline__ FF ff_mac(FF acc, float m, FF u) {
+  const FF p = two_prod(m, u.hi);
+  const FF s = two_sum(acc.hi, p.hi);
+  return FF{s.hi, s.lo + (acc.lo + fmaf(m, u.lo, p.lo))};
+}
+__device__ __forceinline__ FF ff_mac(FF acc, FF m, float u) { return ff_mac(acc, u, m); }
+
+// 1 / b and sqrt(b) by one Newton step from the float value
+__device__ __forceinline__ FF ff_recip(FF b) {
+  const float r = 1.f / b.hi;
+  const float e = fmaf(-b.lo, r, fmaf(-b.hi, r, 1.f));
+  return fast_two_sum(r, r * e);
+}
+__device__ __forceinline__ FF ff_sqrt(FF b) {
+  const float h = sqrtf(b.hi);
+  const float e = fmaf(-h, h, b.hi) + b.lo;
+  return fast_two_sum(h, e * (0.5f / h));
 }
 
-// a times a small integer k (|k| <= 6): exact in float-float
-__device__ __forceinline__ FF ff_scale(FF a, float k) {
-  const float p = a.hi * k;
-  return fast_two_sum(p, fmaf(a.hi, k, -p) + a.lo * k);
-}
-
-// a + t (b + t (c + t d)) in float-float, rounded to float
-__device__ __forceinline__ float ff_horner3(FF t, FF a, FF b, FF c, FF d) {
-  FF r = ff_add(ff_mul(d, t), c);
-  r = ff_add(ff_mul(r, t), b);
-  r = ff_add(ff_mul(r, t), a);
-  return r.hi + r.lo;
-}
-
-// The moments of float populations (deviations d_i for half storage, with the weights' own moments
-// times c added) for the fields readout: per direction pair, the sums over energies for +v and -v
-// are first combined into their sum P and difference D, and the moments accumulate c P (even
-// moments) and c D (odd moments) in float.  The odd moments (the velocity) then cancel within each
-// direction pair before they are summed over directions, which keeps T^{0a} near float rounding of
-// the populations (about 1e-8 of T^00; summing +v and -v over all directions first and subtracting
-// at the end loses an order of magnitude more).  Returned in double, with the weights' own moments
-// and T^zz (trace identity) added in double.
+// The moments of float populations (deviations d_i for half storage) for the fields readout: per
+// direction pair, the sums over energies for +v and -v are first combined into their sum P and
+// difference D, and the moments accumulate c P (even moments) and c D (odd moments) in float.  The
+// odd moments (the velocity) then cancel within each direction pair before they are summed over
+// directions, which keeps T^{0a} near float rounding of the populations (about 1e-8 of T^00; summing
+// +v and -v over all directions first and subtracting at the end loses an order of magnitude more).
+// T^zz is left 0; moments_ext adds it and the weights' own moments.
 template <class L, bool DEV, class GetF>
-__device__ __forceinline__ Mom<double> moments_pd(GetF&& getf, double c) {
+__device__ __forceinline__ Mom<float> moments_pd(GetF&& getf) {
   float N0 = 0.f, Nx = 0.f, Ny = 0.f, Nz = 0.f, T00 = 0.f, T0x = 0.f, T0y = 0.f, T0z = 0.f, Txx = 0.f, Tyy = 0.f,
         Txy = 0.f, Txz = 0.f, Tyz = 0.f;
   static_for<L::NDP>([&](auto K) {
@@ -1177,22 +1248,140 @@ __device__ __forceinline__ Mom<double> moments_pd(GetF&& getf, double c) {
     if constexpr (vx != 0 && vz != 0) Txz = fmaf((float)(vx * vz * ir2), P2, Txz);
     if constexpr (vy != 0 && vz != 0) Tyz = fmaf((float)(vy * vz * ir2), P2, Tyz);
   });
-  Mom<double> m{N0, Nx, Ny, Nz, T00, T0x, T0y, T0z, Txx, Tyy, 0.0, Txy, Txz, Tyz};
-  if constexpr (DEV) add_rest_sums<L, double>(m, c);
-  m.Tzz = m.T00 - m.Txx - m.Tyy;
-  return m;
+  return Mom<float>{N0, Nx, Ny, Nz, T00, T0x, T0y, T0z, Txx, Tyy, 0.f, Txy, Txz, Tyz};
 }
 
+// The float sums completed in float-float: the weights' own moments times c (deviations), and T^zz
+// from the trace identity.  Without deviations every moment but T^zz is its float sum exactly.
+template <bool DEV>
+struct MomExt {
+  using M = std::conditional_t<DEV, FF, float>;
+  M N0, T00, Txx, Tyy, Txy, Txz, Tyz;
+  float Nx, Ny, Nz, T0x, T0y, T0z;  // odd moments: the weights' own vanish
+  FF Tzz;
+};
+template <class L, bool DEV>
+__device__ __forceinline__ MomExt<DEV> moments_ext(const Mom<float>& m, float c) {
+  MomExt<DEV> r;
+  r.Nx = m.Nx, r.Ny = m.Ny, r.Nz = m.Nz, r.T0x = m.T0x, r.T0y = m.T0y, r.T0z = m.T0z;
+  if constexpr (DEV) {
+    using W = RestSums<L>;
+    auto add = [&](double w, float v) { return ff_add(ff_mul(ff_const(w), c), v); };
+    r.N0 = add(W::N0, m.N0), r.T00 = add(W::T00, m.T00), r.Txx = add(W::Txx, m.Txx), r.Tyy = add(W::Tyy, m.Tyy);
+    r.Txy = add(W::Txy, m.Txy), r.Txz = add(W::Txz, m.Txz), r.Tyz = add(W::Tyz, m.Tyz);
+    r.Tzz = ff_sub(r.T00, ff_add(r.Txx, r.Tyy));
+  } else {
+    r.N0 = m.N0, r.T00 = m.T00, r.Txx = m.Txx, r.Tyy = m.Tyy, r.Txy = m.Txy, r.Txz = m.Txz, r.Tyz = m.Tyz;
+    const FF s = two_sum(m.Txx, m.Tyy);
+    r.Tzz = ff_add(ff_neg(s), m.T00);
+  }
+  return r;
+}
+__device__ __forceinline__ double to_double(float x) { return (double)x; }
+__device__ __forceinline__ double to_double(FF x) { return ff_double(x); }
+__device__ __forceinline__ float to_float(float x) { return x; }
+__device__ __forceinline__ float to_float(FF x) { return x.hi; }
+template <class To, bool DEV>
+__device__ __forceinline__ Mom<To> mom_of(const MomExt<DEV>& m) {
+  auto t = [](auto v) -> To {
+    if constexpr (std::is_same<To, double>::value) return to_double(v);
+    else return to_float(v);
+  };
+  return Mom<To>{t(m.N0),  t(m.Nx),  t(m.Ny),  t(m.Nz),  t(m.T00), t(m.T0x), t(m.T0y),
+                 t(m.T0z), t(m.Txx), t(m.Tyy), t(m.Tzz), t(m.Txy), t(m.Txz), t(m.Tyz)};
+}
+
+// One update of a converged float Landau frame against the float-float moments.  With U made a unit
+// vector to float-float precision, V = T.(eta U), eps = U.V and the residual r = V - eps U (orthogonal
+// to U), the shifted power update (see landau_from) is U + 3 r / (4 eps) to second order in r: one
+// product with T in extended precision, and the update itself, some 1e-7 U, needs float only.  The
+// second-order terms of the norm and of the Rayleigh quotient are added (d.d is minus the square of
+// the update).  The same update in double took 60 % of the fields kernel at the 1/64-rate double pipe.
+struct FrameFF {
+  FF U0, Ux, Uy, Uz, eps, n;
+  bool ok;
+};
+template <bool DEV>
+__device__ __forceinline__ FrameFF frame_update(const MomExt<DEV>& m, const Landau<float>& lf) {
+  const FF z{0.f, 0.f};
+  const float x = lf.Ux, y = lf.Uy, w = lf.Uz;
+  FF q = ff_mac(ff_mac(ff_mac(FF{1.f, 0.f}, x, x), y, y), w, w);
+  const FF U0 = ff_sqrt(fast_two_sum(q.hi, q.lo));
+  auto row = [&](auto a, auto b, auto c, auto d) {
+    const FF r = ff_mac(ff_mac(ff_mac(ff_mac(z, a, U0), b, -x), c, -y), d, -w);
+    return fast_two_sum(r.hi, r.lo);
+  };
+  const FF V0 = row(m.T00, m.T0x, m.T0y, m.T0z), Vx = row(m.T0x, m.Txx, m.Txy, m.Txz);
+  const FF Vy = row(m.T0y, m.Txy, m.Tyy, m.Tyz), Vz = row(m.T0z, m.Txz, m.Tyz, m.Tzz);
+  FF e = ff_mac(ff_mac(ff_mac(ff_mac(z, V0, U0), Vx, -x), Vy, -y), Vz, -w);
+  e = fast_two_sum(e.hi, e.lo);
+  const float k = 0.75f / e.hi;
+  auto res = [&](FF V, FF u) {  // k (V - e u): V and e u agree to float rounding, so the difference is exact
+    const FF p = ff_mul(e, u);
+    return k * ((V.hi - p.hi) + (V.lo - p.lo));
+  };
+  float d0 = res(V0, U0), dx = res(Vx, FF{x, 0.f}), dy = res(Vy, FF{y, 0.f}), dz = res(Vz, FF{w, 0.f});
+  const float dd = d0 * d0 - dx * dx - dy * dy - dz * dz;
+  const float h = -0.5f * dd;
+  FrameFF r;
+  r.U0 = ff_add(U0, fmaf(h, U0.hi, d0));
+  r.Ux = two_sum(x, fmaf(h, x, dx));
+  r.Uy = two_sum(y, fmaf(h, y, dy));
+  r.Uz = two_sum(w, fmaf(h, w, dz));
+  r.eps = ff_add(e, (float)(4.0 / 3.0) * dd * e.hi);
+  FF nn = ff_mac(z, m.N0, r.U0);
+  nn = ff_mac(nn, -m.Nx, r.Ux);
+  nn = ff_mac(nn, -m.Ny, r.Uy);
+  nn = ff_mac(nn, -m.Nz, r.Uz);
+  r.n = fast_two_sum(nn.hi, nn.lo);
+  r.ok = r.eps.hi > 0.f && r.n.hi > 0.f && isfinite(r.eps.hi) && isfinite(r.n.hi);
+  return r;
+}
+
+// Block sums of d[0..4] over kMomThreads threads into out[0..4].  The warps' five sums are reduced
+// together: at each of the first three exchanges a lane keeps half of what it holds and hands its
+// partner the rest, so a warp adds 8 doubles a lane instead of 25 (the same pairs in the same tree
+// as a shuffle reduction of each value).
+__device__ __forceinline__ void block_sums(const double (&d)[5], double* __restrict__ out) {
+  __shared__ double ws[kMomThreads / 32][8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+  auto swap = [](double keep, double give, int o) { return keep + __shfl_xor_sync(0xffffffffu, give, o); };
+  // lanes with bit 4 clear take values 0, 1, 2, the others 3, 4 (and a zero)
+  const double e0 = swap(b4 ? d[3] : d[0], b4 ? d[0] : d[3], 16);
+  const double e1 = swap(b4 ? d[4] : d[1], b4 ? d[1] : d[4], 16);
+  const double e2 = swap(b4 ? 0.0 : d[2], b4 ? d[2] : 0.0, 16);
+  // bit 3 clear: the first two of those, set: the third
+  const double g0 = swap(b3 ? e2 : e0, b3 ? e0 : e2, 8);
+  const double g1 = swap(b3 ? 0.0 : e1, b3 ? e1 : 0.0, 8);
+  // bit 2 clear: the first, set: the second
+  double h = swap(b2 ? g1 : g0, b2 ? g0 : g1, 4);
+  h += __shfl_xor_sync(0xffffffffu, h, 2);
+  h += __shfl_xor_sync(0xffffffffu, h, 1);
+  if ((lane & 3) == 0) ws[warp][lane >> 2] = h;  // lane 0, 4, 8, 16, 20: values 0, 1, 2, 3, 4
+  __syncthreads();
+  if (threadIdx.x < 5) {
+    const int k = threadIdx.x < 3 ? threadIdx.x : threadIdx.x + 1;
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < kMomThreads / 32; ++w) s += ws[w][k];
+    out[threadIdx.x] = s;
+  }
+}
+
+// The double solve of a float readout, out of line like the step's (few cells take it).
+static __device__ __noinline__ Landau<double> landau_readout_fp64(const Mom<double> m) { return landau<double, 200>(m); }
+
 // ---------------------------------------------------------------------------------------------
-// fields and conserved densities of one time level (double arithmetic; for float storages the
-// Landau solve starts from the float solution and stops at 1e-12 U0)
-//   PULL = true : the pre-collision populations pulled from the previous state (GENERAL: modulo
-//                 wrap, for periodic axes shorter than the stencil reach)
+// fields and conserved densities of one time level.  Double storage: double moments and Landau solve.
+// Float storages: float moments (moments_pd), the step's Landau policy, and one update of a float
+// frame in float-float (frame_update).
+//   PULL = true : the pre-collision populations pulled from the previous state
 //   PULL = false: the stored populations of each cell
 // out.f[k][cell], k = n, eps, U0, U1, U2, U3; partial[block][5] = block sums of
-// N^0, T^00, T^0x, T^0y, T^0z, reduced by warp shuffles in a fixed order.
+// N^0, T^00, T^0x, T^0y, T^0z, in a fixed order.
 // ---------------------------------------------------------------------------------------------
-template <class L, class S, bool PULL, bool GENERAL>
+template <class L, class S, bool PULL, bool WALLS>
 __global__ void __launch_bounds__(kMomThreads) k_fields(const typename S::T* __restrict__ src,
                                                         const __grid_constant__ StepParams p,
                                                         const FieldOut out,
@@ -1204,79 +1393,155 @@ __global__ void __launch_bounds__(kMomThreads) k_fields(const typename S::T* __r
   const int gid = blk * kMomThreads + threadIdx.x;
   const bool valid = gid < p.cells;
   const Cell cl = make_cell(valid ? gid : p.cells - 1, p);
+  const PullTab<L> tab(cl, p);
   auto index = [&](auto I) -> long long {
     constexpr int i = decltype(I)::value;
-    return PULL ? pull_index<L, i, GENERAL, true>(cl, p) : (long long)i * p.cells + cl.c;
+    if constexpr (PULL) return tab.template index<i, WALLS>(cl, p);
+    else return (long long)i * p.cells + (unsigned)cl.c;
   };
-  Mom<double> m;
-  Landau<double> lw;
+  double d[5];
+  bool ok, finite;
+  double n, eps, U0, Ux, Uy, Uz;
+  auto put = [&](const Landau<double>& lw) {
+    ok = lw.ok;
+    n = lw.n, eps = lw.eps, U0 = lw.U0, Ux = lw.Ux, Uy = lw.Uy, Uz = lw.Uz;
+  };
+  auto all_finite = [](const auto& m) {
+    return isfinite(m.N0) && isfinite(m.Nx) && isfinite(m.Ny) && isfinite(m.Nz) && isfinite(m.T00) &&
+           isfinite(m.T0x) && isfinite(m.T0y) && isfinite(m.T0z) && isfinite(m.Txx) && isfinite(m.Tyy) &&
+           isfinite(m.Tzz) && isfinite(m.Txy) && isfinite(m.Txz) && isfinite(m.Tyz);
+  };
   if constexpr (std::is_same<typename S::A, double>::value) {
-    m = moments<L, double>([&](auto I) -> double { return src[index(I)]; });
-    lw = landau<double, 200>(m);
+    const Mom<double> m = moments<L, double>([&](auto I) -> double { return src[index(I)]; });
+    put(landau<double, 200>(m));
+    finite = all_finite(m);
+    d[0] = m.N0, d[1] = m.T00, d[2] = m.T0x, d[3] = m.T0y, d[4] = m.T0z;
   } else {
-    // float populations: the per-cell moments in float with each direction pair's difference taken
-    // first (moments_pd; deviations for half storage); the cross-cell sums below in double
     constexpr bool DEV = std::is_same<S, StoreF16Dev>::value;
-    auto getf = [&](auto I) -> float {
-      constexpr int i = decltype(I)::value;
-      if constexpr (DEV) return S::template load_dev<L, i>(src + index(I), p);
-      else return (float)src[index(I)];
-    };
-    m = moments_pd<L, DEV>(getf, (double)p.half_nref);
+    const MomExt<DEV> m = moments_ext<L, DEV>(
+        moments_pd<L, DEV>([&](auto I) -> float {
+          constexpr int i = decltype(I)::value;
+          if constexpr (DEV) return S::template load_dev<L, i>(src + index(I), p);
+          else return __ldcg(src + index(I));
+        }),
+        p.half_nref);
     // the step's policy: float solve, double for cells above gamma_thr, for unconverged float
-    // solves, or everywhere with landau_fp64; the result of a float solve is refined by one
-    // double update (n and eps are the double Rayleigh quotients of the float U)
-    const Mom<float> mf = convert<double, float>(m);
+    // solves, or everywhere with landau_fp64
+    const Mom<float> mf = mom_of<float>(m);
+    finite = all_finite(mf);
     const float NN = mf.N0 * mf.N0 - mf.Nx * mf.Nx - mf.Ny * mf.Ny - mf.Nz * mf.Nz;
     bool dbl = p.landau_fp64 || mf.N0 * mf.N0 > p.gamma_thr2 * NN;
     if (!dbl) {
       const Landau<float> lf = landau<float, 8>(mf);
-      if (lf.ok && lf.conv)
-        lw = landau_from<double, 1>(m, (double)lf.U0, (double)lf.Ux, (double)lf.Uy, (double)lf.Uz, 1e-10);
       dbl = !(lf.ok && lf.conv);
+      if (!dbl) {
+        const FrameFF r = frame_update<DEV>(m, lf);
+        ok = r.ok;
+        n = ff_double(r.n), eps = ff_double(r.eps);
+        U0 = ff_double(r.U0), Ux = ff_double(r.Ux), Uy = ff_double(r.Uy), Uz = ff_double(r.Uz);
+      }
     }
-    if (dbl) lw = landau<double, 200>(m);
+    if (dbl) put(landau_readout_fp64(mom_of<double>(m)));
+    d[0] = to_double(m.N0), d[1] = to_double(m.T00), d[2] = m.T0x, d[3] = m.T0y, d[4] = m.T0z;
   }
   if (valid) {
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
-    out.f[0][cl.c] = lw.ok ? lw.n : nan;
-    out.f[1][cl.c] = lw.ok ? lw.eps : nan;
-    out.f[2][cl.c] = lw.ok ? lw.U0 : nan;
-    out.f[3][cl.c] = lw.ok ? lw.Ux : nan;
-    out.f[4][cl.c] = lw.ok ? lw.Uy : nan;
-    out.f[5][cl.c] = lw.ok ? lw.Uz : nan;
+    out.f[0][cl.c] = ok ? n : nan;
+    out.f[1][cl.c] = ok ? eps : nan;
+    out.f[2][cl.c] = ok ? U0 : nan;
+    out.f[3][cl.c] = ok ? Ux : nan;
+    out.f[4][cl.c] = ok ? Uy : nan;
+    out.f[5][cl.c] = ok ? Uz : nan;
     // non-finite populations show as non-finite moments; any other cell without a frame is a
     // Landau failure
-    const bool finite = isfinite(m.N0) && isfinite(m.Nx) && isfinite(m.Ny) && isfinite(m.Nz) && isfinite(m.T00) &&
-                        isfinite(m.T0x) && isfinite(m.T0y) && isfinite(m.T0z) && isfinite(m.Txx) &&
-                        isfinite(m.Tyy) && isfinite(m.Tzz) && isfinite(m.Txy) && isfinite(m.Txz) && isfinite(m.Tyz);
     if (!finite) atomicAdd(&status[kStatusNan], 1);
-    else if (!lw.ok) atomicAdd(&status[kStatusNonconv], 1);
+    else if (!ok) atomicAdd(&status[kStatusNonconv], 1);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) d[k] = 0.0;
   }
-  double d[5] = {valid ? m.N0 : 0.0, valid ? m.T00 : 0.0, valid ? m.T0x : 0.0, valid ? m.T0y : 0.0,
-                 valid ? m.T0z : 0.0};
+  block_sums(d, partial + (long long)blk * 5);
+}
+
+// Second pass of the conserved-density sums, value blockIdx.x of the five: one block adds the
+// per-block partials in a fixed order (thread t takes blocks t, t + 256, ...; then a shuffle and
+// shared-memory tree), so the totals are bitwise reproducible.  The adds of a thread are a chain; its
+// loads are not, so 16 are kept in flight.
+static __global__ void __launch_bounds__(kReduceThreads) k_reduce_partials(const double* __restrict__ partial,
+                                                                           int nblocks, double* __restrict__ totals) {
+  __shared__ double ws[kReduceThreads / 32];
+  const int k = blockIdx.x;
+  double d = 0.0;
+#pragma unroll 16
+  for (int b = threadIdx.x; b < nblocks; b += kReduceThreads) d += partial[(long long)b * 5 + k];
 #pragma unroll
-  for (int k = 0; k < 5; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d[k] += __shfl_down_sync(0xffffffffu, d[k], o);
-  __shared__ double ws[kMomThreads / 32][5];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < 5; ++k) ws[warp][k] = d[k];
+  for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = d;
   __syncthreads();
-  if (threadIdx.x < 5) {
+  if (threadIdx.x == 0) {
     double s = 0.0;
 #pragma unroll
-    for (int w = 0; w < kMomThreads / 32; ++w) s += ws[w][threadIdx.x];
-    partial[(long long)blk * 5 + threadIdx.x] = s;
+    for (int w = 0; w < kReduceThreads / 32; ++w) s += ws[w];
+    totals[k] = s;
   }
 }
 
 // ---------------------------------------------------------------------------------------------
-// initial state f_i = f_i^eq(n, T, u) (per-level form: coefficients in double, Horner steps in the
-// storage's arithmetic), and population format conversion
+// initial state f_i = f_i^eq(n, T, u), and population format conversion
 // ---------------------------------------------------------------------------------------------
+// The equilibrium's coefficients per energy level (eq_coef and level_coef) in float-float.
+template <class L>
+__device__ __forceinline__ LevCoef<L, FF> level_coef_ff(FF n, FF T, FF x) {
+  LevCoef<L, FF> r;
+  const FF x2 = ff_mul(x, x), T2 = ff_mul(T, T);
+  const FF nT = ff_mul(n, ff_recip(T));
+  auto times = [](FF a, float k) { return ff_mul(a, k); };
+  if constexpr (L::ORDER == 3) {
+    const FF pref = ff_mul(ff_const(1.0 / 12.0), nT);
+    const FF nTh = ff_scale2(nT, 0.5f), nTq = ff_scale2(nT, 0.25f);  // 6 pref, 3 pref
+    const FF Tn = ff_mul(nTh, T);                                     // 6 pref T
+    // c00 = -6 pref (x2 (8x + 4) + (4x - 2) + T2 (1 - 4x)), ...
+    const FF x4 = ff_scale2(x, 4.f), x6 = times(x, 6.f);
+    FF c00 = ff_add(ff_mul(x2, ff_add(ff_scale2(x, 8.f), 4.f)), ff_add(x4, -2.f));
+    c00 = ff_neg(ff_mul(nTh, ff_add(c00, ff_mul(T2, ff_add(ff_neg(x4), 1.f)))));
+    FF c10 = ff_add(ff_mul(x2, ff_add(ff_scale2(x6, 2.f), 8.f)), ff_add(times(x, 5.f), -1.f));
+    c10 = ff_mul(nTh, ff_add(c10, ff_mul(T2, ff_add(ff_neg(x6), 1.f))));
+    const FF c01 = ff_mul(Tn, ff_sub(ff_add(times(x2, 12.f), 3.f), ff_scale2(T2, 2.f)));
+    FF c20 = ff_add(ff_mul(x, ff_add(x6, 3.f)), 2.f);
+    c20 = ff_neg(ff_mul(ff_mul(nTq, x), ff_sub(c20, ff_scale2(T2, 2.f))));
+    const FF c11 = ff_neg(ff_mul(Tn, ff_sub(ff_add(ff_mul(x, ff_add(x6, 1.f)), 1.f), T2)));
+    const FF c02 = ff_neg(ff_mul(ff_mul(nTq, T2), ff_add(x6, -1.f)));
+    const FF px = ff_mul(pref, x), px2 = ff_mul(px, x), pT2 = ff_mul(pref, T2);
+    const FF a3 = ff_mul(px2, x), b3 = times(ff_mul(px2, T), 3.f), c3 = times(ff_mul(px, T2), 3.f), d3 = ff_mul(pT2, T);
+    static_for<L::NLEV>([&](auto K) {
+      constexpr int l = decltype(K)::value;
+      constexpr double pd = L::P0[l];
+      const FF p = ff_const(pd), p2 = ff_const(pd * pd), p3 = ff_const(pd * pd * pd);
+      r.a[l] = ff_add(ff_add(c00, ff_mul(p, c10)), ff_add(ff_mul(p2, c20), ff_mul(p3, a3)));
+      r.b[l] = ff_add(ff_mul(p, c01), ff_add(ff_mul(p2, c11), ff_mul(p3, b3)));
+      r.c[l] = ff_add(ff_mul(p2, c02), ff_mul(p3, c3));
+      r.d[l] = ff_mul(p3, d3);
+    });
+  } else {
+    const FF pref = ff_scale2(nT, 0.25f), nTh = ff_scale2(nT, 0.5f), Tn = ff_mul(nTh, T);  // pref, 2 pref, 2 pref T
+    const FF x4 = ff_scale2(x, 4.f);
+    const FF c00 = ff_mul(nTh, ff_sub(ff_add(ff_scale2(x2, 4.f), 2.f), T2));
+    const FF c10 = ff_neg(ff_mul(nTh, ff_sub(ff_add(ff_mul(x, ff_add(x4, 1.f)), 1.f), T2)));
+    const FF c01 = ff_neg(ff_mul(Tn, ff_add(x4, -1.f)));
+    const FF px = ff_mul(pref, x), a2 = ff_mul(px, x), b2 = ff_scale2(ff_mul(px, T), 2.f), c2 = ff_mul(pref, T2);
+    static_for<L::NLEV>([&](auto K) {
+      constexpr int l = decltype(K)::value;
+      constexpr double pd = L::P0[l];
+      const FF p = ff_const(pd), p2 = ff_const(pd * pd);
+      r.a[l] = ff_add(c00, ff_add(ff_mul(p, c10), ff_mul(p2, a2)));
+      r.b[l] = ff_add(ff_mul(p, c01), ff_mul(p2, b2));
+      r.c[l] = ff_mul(p2, c2);
+      r.d[l] = FF{0.f, 0.f};
+    });
+  }
+  return r;
+}
+
 template <class L, class S>
 __global__ void __launch_bounds__(128) k_init(const double* __restrict__ n, const double* __restrict__ Tf,
                                               const double* __restrict__ u, typename S::T* __restrict__ dst,
@@ -1295,9 +1560,9 @@ __global__ void __launch_bounds__(128) k_init(const double* __restrict__ n, cons
   }
   const double g = rsqrt(1.0 - u2);
   const double Ux = g * ux, Uy = g * uy, Uz = g * uz;
-  // the equilibrium per energy level (see level_coef), coefficients in double
-  const LevCoef<L, double> ed = level_coef<L, double>(eq_coef<L::ORDER, double>(nn, T, g));
   if constexpr (std::is_same<typename S::A, double>::value) {
+    // the equilibrium per energy level (see level_coef), coefficients in double
+    const LevCoef<L, double> ed = level_coef<L, double>(eq_coef<L::ORDER, double>(nn, T, g));
     static_for<L::NDP>([&](auto K) {
       constexpr int k = decltype(K)::value;
       constexpr int first = L::DP_FIRST[k];
@@ -1317,35 +1582,61 @@ __global__ void __launch_bounds__(128) k_init(const double* __restrict__ n, cons
   } else {
     // Float storage rounds every population to float.  The cubic in t cancels strongly at the high
     // energy levels (terms up to ~200 times the value at p0 = 10.95, |u| = 0.6), so those levels
-    // (p0 > 4) are evaluated in float-float arithmetic (a value as an unevaluated sum hi + lo of
-    // two floats; error-free sums and products by FMA), the others in float: every population ends
-    // within float rounding of the double evaluation, with no double arithmetic per population.
-    LevCoef<L, FF> e;
-    static_for<L::NLEV>([&](auto K) {
-      constexpr int l = decltype(K)::value;
-      e.a[l] = ff_from(ed.a[l]);
-      e.b[l] = ff_from(ed.b[l]);
-      e.c[l] = ff_from(ed.c[l]);
-      e.d[l] = ff_from(ed.d[l]);
-    });
-    const FF Uxf = ff_from(Ux), Uyf = ff_from(Uy), Uzf = ff_from(Uz);
+    // (p0 > 4) are evaluated with the rounding errors of their products and sums carried along
+    // (compensated; the even part a + c t^2 and the odd part t (b + d t^2) shared by +v and -v), the
+    // others in float: every population ends within float rounding of the double evaluation.  The
+    // inputs are normalised in double (some 40 operations a cell, which the 1/64-rate pipe does
+    // beside the float work); the coefficients, 110 double operations a cell and the bound of this
+    // kernel while they were double, are float-float.
+    const LevCoef<L, FF> e = level_coef_ff<L>(ff_from(nn), ff_from(T), ff_from(fma(T, g, -1.0)));
+    // U / R times 1 .. 6 per axis: t = v.U / R is then a sum of at most three of them
+    FF m[3][7];
+    const double Ua[3] = {Ux * L::INV_R, Uy * L::INV_R, Uz * L::INV_R};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      m[a][1] = ff_from(Ua[a]);
+      m[a][3] = ff_mul(m[a][1], 3.f);
+      m[a][5] = ff_mul(m[a][1], 5.f);
+      m[a][2] = ff_scale2(m[a][1], 2.f);
+      m[a][4] = ff_scale2(m[a][1], 4.f);
+      m[a][6] = ff_scale2(m[a][3], 2.f);
+    }
     static_for<L::NDP>([&](auto K) {
       constexpr int k = decltype(K)::value;
       constexpr int first = L::DP_FIRST[k];
       constexpr int np = L::DP_NPAIR[k];
-      constexpr int vx = L::VX[first], vy = L::VY[first], vz = L::VZ[first];
-      // t = v.U / R: exact small-integer multiples, float-float sum and scaling
-      const FF t = ff_mul(ff_add(ff_add(ff_scale(Uxf, (float)vx), ff_scale(Uyf, (float)vy)), ff_scale(Uzf, (float)vz)),
-                          ff_from(L::INV_R));
+      constexpr int v[3] = {L::VX[first], L::VY[first], L::VZ[first]};
+      static_assert(L::VMAX_X <= 6 && L::VMAX_Y <= 6 && L::VMAX_Z <= 6, "multiples of U up to 6");
+      FF t{0.f, 0.f};
+      static_for<3>([&](auto A) {
+        constexpr int a = decltype(A)::value, va = v[a] < 0 ? -v[a] : v[a];
+        if constexpr (va != 0) {
+          const FF x = v[a] < 0 ? ff_neg(m[a][va]) : m[a][va];
+          const FF s = two_sum(t.hi, x.hi);
+          t = FF{s.hi, s.lo + (t.lo + x.lo)};
+        }
+      });
+      const float t2h = __fmul_rn(t.hi, t.hi);
+      const float t2l = fmaf(2.f * t.hi, t.lo, fmaf(t.hi, t.hi, -t2h));
       static_for<np>([&](auto J) {
         constexpr int ip = first + 2 * decltype(J)::value;
         constexpr int l = L::LEV[ip];
         constexpr float w = (float)L::W[ip];
         float Ep, Em;
         if constexpr (L::P0[l] > 4.0) {
-          const FF tm = ff_neg(t);
-          Ep = ff_horner3(t, e.a[l], e.b[l], e.c[l], e.d[l]);
-          Em = ff_horner3(tm, e.a[l], e.b[l], e.c[l], e.d[l]);
+          auto lin = [&](FF c0, FF c1) {  // c0 + c1 t^2
+            const FF q = two_prod(c1.hi, t2h);
+            const FF s = two_sum(c0.hi, q.hi);
+            return FF{s.hi, s.lo + fmaf(c1.hi, t2l, fmaf(c1.lo, t2h, c0.lo + q.lo))};
+          };
+          const FF even = lin(e.a[l], e.c[l]);
+          FF b = e.b[l];
+          if constexpr (L::ORDER == 3) b = lin(e.b[l], e.d[l]);
+          FF odd = two_prod(b.hi, t.hi);
+          odd.lo += fmaf(b.hi, t.lo, b.lo * t.hi);
+          const FF sp = two_sum(even.hi, odd.hi), sm = two_sum(even.hi, -odd.hi);
+          Ep = sp.hi + (sp.lo + (even.lo + odd.lo));
+          Em = sm.hi + (sm.lo + (even.lo - odd.lo));
         } else {
           const float tf = t.hi + t.lo;
           Ep = fmaf(tf, fmaf(tf, fmaf(tf, e.d[l].hi, e.c[l].hi), e.b[l].hi), e.a[l].hi);

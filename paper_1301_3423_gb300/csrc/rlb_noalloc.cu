@@ -38,60 +38,26 @@ __global__ void __launch_bounds__(kMomThreads) k_densities_noalloc(const typenam
   // per-cell moments in the arithmetic rlb_moments uses for this storage (double for double
   // populations; the fields kernel's float sums for float and half-deviation ones), summed across
   // cells in double
-  Mom<double> m;
+  double d[5];
   if constexpr (std::is_same<typename S::A, double>::value) {
-    m = moments<L, double>([&](auto I) -> double { return src[(long long)decltype(I)::value * p.cells + c]; });
+    const Mom<double> m = moments<L, double>([&](auto I) -> double { return src[(long long)decltype(I)::value * p.cells + c]; });
+    d[0] = m.N0, d[1] = m.T00, d[2] = m.T0x, d[3] = m.T0y, d[4] = m.T0z;
   } else {
     constexpr bool DEV = std::is_same<S, StoreF16Dev>::value;
-    auto getf = [&](auto I) -> float {
-      constexpr int i = decltype(I)::value;
-      if constexpr (DEV) return S::template load_dev<L, i>(src + (long long)i * p.cells + c, p);
-      else return (float)src[(long long)i * p.cells + c];
-    };
-    m = moments_pd<L, DEV>(getf, (double)p.half_nref);
+    const MomExt<DEV> m = moments_ext<L, DEV>(
+        moments_pd<L, DEV>([&](auto I) -> float {
+          constexpr int i = decltype(I)::value;
+          if constexpr (DEV) return S::template load_dev<L, i>(src + (long long)i * p.cells + c, p);
+          else return (float)src[(long long)i * p.cells + c];
+        }),
+        p.half_nref);
+    d[0] = to_double(m.N0), d[1] = to_double(m.T00), d[2] = m.T0x, d[3] = m.T0y, d[4] = m.T0z;
   }
-  double d[5] = {valid ? m.N0 : 0.0, valid ? m.T00 : 0.0, valid ? m.T0x : 0.0, valid ? m.T0y : 0.0,
-                 valid ? m.T0z : 0.0};
+  if (!valid) {
 #pragma unroll
-  for (int k = 0; k < 5; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d[k] += __shfl_down_sync(0xffffffffu, d[k], o);
-  __shared__ double ws[kMomThreads / 32][5];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < 5; ++k) ws[warp][k] = d[k];
-  __syncthreads();
-  if (threadIdx.x < 5) {
-    double s = 0.0;
-#pragma unroll
-    for (int w = 0; w < kMomThreads / 32; ++w) s += ws[w][threadIdx.x];
-    partial[(long long)blockIdx.x * 5 + threadIdx.x] = s;
+    for (int k = 0; k < 5; ++k) d[k] = 0.0;
   }
-}
-
-// Second pass: one block adds the partials in a fixed order and writes the 5 totals.
-__global__ void __launch_bounds__(kReduceThreads) k_totals_noalloc(const double* __restrict__ partial, int nblocks,
-                                                                    double* __restrict__ totals) {
-  __shared__ double ws[kReduceThreads / 32][5];
-  double d[5] = {0, 0, 0, 0, 0};
-  for (int b = threadIdx.x; b < nblocks; b += kReduceThreads)
-#pragma unroll
-    for (int k = 0; k < 5; ++k) d[k] += partial[(long long)b * 5 + k];
-#pragma unroll
-  for (int k = 0; k < 5; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d[k] += __shfl_down_sync(0xffffffffu, d[k], o);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < 5; ++k) ws[warp][k] = d[k];
-  __syncthreads();
-  if (threadIdx.x < 5) {
-    double s = 0.0;
-    for (int w = 0; w < kReduceThreads / 32; ++w) s += ws[w][threadIdx.x];
-    totals[threadIdx.x] = s;
-  }
+  block_sums(d, partial + (long long)blockIdx.x * 5);
 }
 
 // Device address of the scratch array, looked up once per device with that device current.
@@ -123,7 +89,7 @@ cudaError_t launch(const void* f, const StepParams& p, double* scratch, int bloc
   k_densities_noalloc<L, S><<<blocks, kMomThreads, 0, s>>>(static_cast<const typename S::T*>(f), p, scratch);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_totals_noalloc<<<1, kReduceThreads, 0, s>>>(scratch, blocks, scratch + (size_t)kNoallocMaxBlocks * 5);
+  k_reduce_partials<<<5, kReduceThreads, 0, s>>>(scratch, blocks, scratch + (size_t)kNoallocMaxBlocks * 5);
   return cudaGetLastError();
 }
 
