@@ -355,6 +355,107 @@ __device__ __forceinline__ Mom<A> moments(Get&& get, A c = A(0)) {
   return m;
 }
 
+// The mirror pairs of each energy level, in order.
+template <class L>
+struct LevelPairs {
+  __host__ __device__ static constexpr int count(int l) {
+    int n = 0;
+    for (int i = 0; i < L::Q; i += 2) n += L::LEV[i] == l;
+    return n;
+  }
+  __host__ __device__ static constexpr int first(int l, int j) {  // the + population of pair j
+    for (int i = 0; i < L::Q; i += 2)
+      if (L::LEV[i] == l && j-- == 0) return i;
+    return -1;
+  }
+  __host__ __device__ static constexpr int sum(int l, int a, int b) {  // of v_a v_b over the pairs
+    int s = 0;
+    for (int i = 0; i < L::Q; i += 2) {
+      const int v[3] = {L::VX[i], L::VY[i], L::VZ[i]};
+      if (L::LEV[i] == l) s += v[a] * v[b];
+    }
+    return s;
+  }
+};
+
+// Moments of double populations, summed in 64-bit integers.  GB300's double pipe retires 2 lanes a
+// clock and SM and bounds the double step; its integer pipe is some 30 times wider.  Per energy level
+// the populations are put on a common grid of 2^-50 to 2^-51 of the level's largest (adding
+// 1.5 2^k leaves the grid value in the low bits of the sum), and the level's sums over v with the
+// integer weights 1, v_a, v_a v_b are exact integers: |v_a v_b| sums to at most 2^11 over the
+// populations, so 51 + 11 bits and the sign fit.  Per level 9 sums return to double and take p0 and
+// p0^2.  The grid is per level, so the rare high levels, which p0^2 weights most, are rounded by their
+// own size: the moments' error is below that of adding the 128 terms in double.  Double operations a
+// cell: 128 adds and 36 conversions, 115 more; 960 when the sums were double.  Integer sums do not
+// depend on their order, so every kernel gets the same bits.
+// Populations that are not finite (or beyond 2^1021, whose moments overflow) give NaN moments.
+template <class L, class Get>
+__device__ __forceinline__ Mom<double> moments_fixed(Get&& get) {
+  using u64 = unsigned long long;
+  Mom<double> m;
+  m.N0 = m.Nx = m.Ny = m.Nz = 0.0;
+  m.T00 = m.T0x = m.T0y = m.T0z = 0.0;
+  m.Txx = m.Tyy = m.Txy = m.Txz = m.Tyz = 0.0;
+  bool finite = true;
+  static_for<L::NLEV>([&](auto K) {
+    constexpr int l = decltype(K)::value;
+    constexpr int n = LevelPairs<L>::count(l);
+    double f[2 * n];
+    unsigned top = 0;
+    static_for<n>([&](auto J) {
+      constexpr int j = decltype(J)::value, i = LevelPairs<L>::first(l, j);
+      f[2 * j] = get(ic<i>{});
+      f[2 * j + 1] = get(ic<i + 1>{});
+      top = max(top, max((unsigned)__double2hiint(f[2 * j]) & 0x7fffffffu,
+                         (unsigned)__double2hiint(f[2 * j + 1]) & 0x7fffffffu));
+    });
+    const int e = max((int)(top >> 20), 64);  // |f| < 2^(e - 1022)
+    finite = finite && e < 2045;
+    const double C = __hiloint2double(((e + 2) << 20) | 0x80000, 0);  // 1.5 2^(e - 1021)
+    const u64 Cb = (u64)__double_as_longlong(C);
+    // sums of the raw bits; each carries a known multiple of those of C, removed below (modulo 2^64)
+    u64 s0 = 0, sxx = 0, syy = 0, sxy = 0, sxz = 0, syz = 0, sx = 0, sy = 0, sz = 0;
+    static_for<n>([&](auto J) {
+      constexpr int j = decltype(J)::value, i = LevelPairs<L>::first(l, j);
+      constexpr int vx = L::VX[i], vy = L::VY[i], vz = L::VZ[i];
+      const u64 a = (u64)__double_as_longlong(__dadd_rn(f[2 * j], C));
+      const u64 b = (u64)__double_as_longlong(__dadd_rn(f[2 * j + 1], C));
+      const u64 sp = a + b, sm = a - b;
+      s0 += sp;
+      if constexpr (vx != 0) sxx += (u64)(long long)(vx * vx) * sp, sx += (u64)(long long)vx * sm;
+      if constexpr (vy != 0) syy += (u64)(long long)(vy * vy) * sp, sy += (u64)(long long)vy * sm;
+      if constexpr (vz != 0) sz += (u64)(long long)vz * sm;
+      if constexpr (vx * vy != 0) sxy += (u64)(long long)(vx * vy) * sp;
+      if constexpr (vx * vz != 0) sxz += (u64)(long long)(vx * vz) * sp;
+      if constexpr (vy * vz != 0) syz += (u64)(long long)(vy * vz) * sp;
+    });
+    auto even = [&](u64 s, int w) { return (double)(long long)(s - (u64)(2ll * w) * Cb); };
+    const double g = __hiloint2double((e - 50) << 20, 0);  // the grid, 2^(e - 1073)
+    const double p1 = L::P0[l] * g, p2 = L::P0[l] * L::P0[l] * g;
+    const double d0 = even(s0, n), dx = (double)(long long)sx, dy = (double)(long long)sy, dz = (double)(long long)sz;
+    m.N0 = fma(p1, d0, m.N0);
+    m.Nx = fma(p1, dx, m.Nx);
+    m.Ny = fma(p1, dy, m.Ny);
+    m.Nz = fma(p1, dz, m.Nz);
+    m.T00 = fma(p2, d0, m.T00);
+    m.T0x = fma(p2, dx, m.T0x);
+    m.T0y = fma(p2, dy, m.T0y);
+    m.T0z = fma(p2, dz, m.T0z);
+    m.Txx = fma(p2, even(sxx, ic<LevelPairs<L>::sum(l, 0, 0)>::value), m.Txx);
+    m.Tyy = fma(p2, even(syy, ic<LevelPairs<L>::sum(l, 1, 1)>::value), m.Tyy);
+    m.Txy = fma(p2, even(sxy, ic<LevelPairs<L>::sum(l, 0, 1)>::value), m.Txy);
+    m.Txz = fma(p2, even(sxz, ic<LevelPairs<L>::sum(l, 0, 2)>::value), m.Txz);
+    m.Tyz = fma(p2, even(syz, ic<LevelPairs<L>::sum(l, 1, 2)>::value), m.Tyz);
+  });
+  m.Nx *= L::INV_R, m.Ny *= L::INV_R, m.Nz *= L::INV_R;
+  m.T0x *= L::INV_R, m.T0y *= L::INV_R, m.T0z *= L::INV_R;
+  m.Txx *= L::INV_R2, m.Tyy *= L::INV_R2, m.Txy *= L::INV_R2, m.Txz *= L::INV_R2, m.Tyz *= L::INV_R2;
+  if (!finite) m.N0 = m.T00 = __longlong_as_double(0x7ff8000000000000ll);
+  // |v|^2 = R^2 for every velocity, so the spatial trace of T equals T^00.
+  m.Tzz = m.T00 - m.Txx - m.Tyy;
+  return m;
+}
+
 template <class A, class B>
 __device__ __forceinline__ Mom<B> convert(const Mom<A>& a) {
   return Mom<B>{B(a.N0),  B(a.Nx),  B(a.Ny),  B(a.Nz),  B(a.T00), B(a.T0x), B(a.T0y),
@@ -432,6 +533,65 @@ __device__ __forceinline__ Landau<A> landau(const Mom<A>& m) {
   return landau_from<A, MAXIT>(m, m.N0 * is, m.Nx * is, m.Ny * is, m.Nz * is, tol);
 }
 
+// Landau matching of double moments.  The power iteration gains one to two digits an update at the
+// relative anisotropies of a flow, some 16 double updates of 50 operations from the Eckart vector.
+// Here the float iteration (whose pipe is 64 times wider) gives U to 1e-7 first; then each correction
+// forms the residual r = V - eps U, V = T.(eta U), in double, and solves (T - eps) d = -r in float: on
+// the vectors orthogonal to U, where r and d live, T - eps is -4 eps / 3 up to the anisotropy, so d is
+// a short Richardson iteration, and U + d is right to the digits that d has (six) beyond the last.
+// Two corrections reach the last place of double.  A cell whose Eckart Lorentz factor exceeds 4 or
+// whose corrections do not fall below 3e-11 U0 takes the power iteration in double (cut off at MAXIT
+// updates).  Out of line: a call keeps the step's code small.
+template <int MAXIT>
+static __device__ __noinline__ Landau<double> landau_f64(const Mom<double> m) {
+  const float N0 = (float)m.N0, Nx = (float)m.Nx, Ny = (float)m.Ny, Nz = (float)m.Nz;
+  const float NN = N0 * N0 - Nx * Nx - Ny * Ny - Nz * Nz;
+  if (N0 > 0.f && 16.f * NN > N0 * N0 && N0 < 1e15f && N0 > 1e-15f) {
+    const Mom<float> t = convert<double, float>(m);
+    const Landau<float> lf = landau<float, 8>(t);
+    if (lf.ok && lf.conv) {
+      double Ux = lf.Ux, Uy = lf.Uy, Uz = lf.Uz;
+      double U0 = sqrt(fma(Ux, Ux, fma(Uy, Uy, fma(Uz, Uz, 1.0))));
+      const float u0 = (float)U0, e1 = lf.eps, k = 0.75f / e1, tiny = 3e-11f * u0;
+      for (int it = 0; it < 4; ++it) {
+        const double V0 = m.T00 * U0 - m.T0x * Ux - m.T0y * Uy - m.T0z * Uz;
+        const double Vx = m.T0x * U0 - m.Txx * Ux - m.Txy * Uy - m.Txz * Uz;
+        const double Vy = m.T0y * U0 - m.Txy * Ux - m.Tyy * Uy - m.Tyz * Uz;
+        const double Vz = m.T0z * U0 - m.Txz * Ux - m.Tyz * Uy - m.Tzz * Uz;
+        const double eps = U0 * V0 - Ux * Vx - Uy * Vy - Uz * Vz;
+        const float r0 = (float)fma(-eps, U0, V0), rx = (float)fma(-eps, Ux, Vx), ry = (float)fma(-eps, Uy, Vy),
+                    rz = (float)fma(-eps, Uz, Vz);
+        float d0 = k * r0, dx = k * rx, dy = k * ry, dz = k * rz;
+        for (int j = 0; j < 12; ++j) {
+          const float g0 = fmaf(t.T00, d0, fmaf(-t.T0x, dx, fmaf(-t.T0y, dy, fmaf(-t.T0z, dz, fmaf(-e1, d0, r0)))));
+          const float gx = fmaf(t.T0x, d0, fmaf(-t.Txx, dx, fmaf(-t.Txy, dy, fmaf(-t.Txz, dz, fmaf(-e1, dx, rx)))));
+          const float gy = fmaf(t.T0y, d0, fmaf(-t.Txy, dx, fmaf(-t.Tyy, dy, fmaf(-t.Tyz, dz, fmaf(-e1, dy, ry)))));
+          const float gz = fmaf(t.T0z, d0, fmaf(-t.Txz, dx, fmaf(-t.Tyz, dy, fmaf(-t.Tzz, dz, fmaf(-e1, dz, rz)))));
+          d0 = fmaf(k, g0, d0), dx = fmaf(k, gx, dx), dy = fmaf(k, gy, dy), dz = fmaf(k, gz, dz);
+          const float step = fmaxf(fmaxf(fabsf(gx), fabsf(gy)), fmaxf(fabsf(gz), fabsf(g0)));
+          const float size = fmaxf(fmaxf(fabsf(dx), fabsf(dy)), fmaxf(fabsf(dz), fabsf(d0)));
+          if (k * step <= 1e-6f * size) break;
+        }
+        U0 += d0, Ux += dx, Uy += dy, Uz += dz;
+        // back to U.U = 1 (to second order in its deviation)
+        const double q = fma(U0, U0, -1.0 - fma(Ux, Ux, fma(Uy, Uy, Uz * Uz)));
+        const double h = -0.5 * q;
+        U0 = fma(h, U0, U0), Ux = fma(h, Ux, Ux), Uy = fma(h, Uy, Uy), Uz = fma(h, Uz, Uz);
+        if (fmaxf(fmaxf(fabsf(dx), fabsf(dy)), fmaxf(fabsf(dz), fabsf(d0))) <= tiny) {
+          Landau<double> r;
+          r.U0 = U0, r.Ux = Ux, r.Uy = Uy, r.Uz = Uz;
+          r.eps = eps;  // of the U before the last correction: second order in it
+          r.n = U0 * m.N0 - Ux * m.Nx - Uy * m.Ny - Uz * m.Nz;
+          r.ok = r.eps > 0.0 && r.n > 0.0 && isfinite(r.eps) && isfinite(r.n);
+          r.conv = true;
+          return r;
+        }
+      }
+    }
+  }
+  return landau<double, MAXIT>(m);
+}
+
 // The double-precision solve of a float step, kept out of line: it runs for few cells and would
 // otherwise grow the step kernel's hot code (a call keeps the caller's register allocation that of
 // the float path).  It starts from the Eckart vector and stops at 1e-12 U0: the populations are
@@ -460,7 +620,7 @@ static __device__ __noinline__ Landau<double> landau_fp64_out_of_line(const Mom<
 template <class A>
 __device__ __forceinline__ Landau<A> landau_step(const Mom<A>& m, const StepParams& p) {
   if constexpr (std::is_same<A, double>::value) {
-    Landau<double> r = landau<double, 40>(m);
+    Landau<double> r = landau_f64<40>(m);
     if (r.ok && !r.conv) {
       const Landau<double> again = landau_from<double, 1>(m, r.U0, r.Ux, r.Uy, r.Uz, 1e-10);
       r.ok = again.ok && again.conv;
@@ -606,20 +766,18 @@ __device__ __forceinline__ void collide(const Landau<A>& lw, A T, A inv_tau, Get
     if constexpr (vx != 0) t = fma(A(vx * ir), lw.Ux, t);
     if constexpr (vy != 0) t = fma(A(vy * ir), lw.Uy, t);
     if constexpr (vz != 0) t = fma(A(vz * ir), lw.Uz, t);
+    const A t2 = t * t;
     const A omp = fma(-t, inv_tau, a), omm = fma(t, inv_tau, a);
     static_for<np>([&](auto J) {
       constexpr int ip = first + 2 * decltype(J)::value;
       constexpr int l = L::LEV[ip];
       constexpr double wd = L::W[ip];
       const A w = A(wd);
-      A Ep, Em;
-      if constexpr (L::ORDER == 3) {
-        Ep = fma(t, fma(t, fma(t, e.d[l], e.c[l]), e.b[l]), e.a[l]);
-        Em = fma(-t, fma(-t, fma(-t, e.d[l], e.c[l]), e.b[l]), e.a[l]);
-      } else {
-        Ep = fma(t, fma(t, e.c[l], e.b[l]), e.a[l]);
-        Em = fma(-t, fma(-t, e.c[l], e.b[l]), e.a[l]);
-      }
+      // the even part a + c t^2 and the odd part's factor b + d t^2 serve both signs of t
+      const A even = fma(t2, e.c[l], e.a[l]);
+      A odd = e.b[l];
+      if constexpr (L::ORDER == 3) odd = fma(t2, e.d[l], odd);
+      const A Ep = fma(t, odd, even), Em = fma(-t, odd, even);
       const A fp = get(ic<ip>{}), fm = get(ic<ip + 1>{});
       if constexpr (DEV) {
         put(ic<ip>{}, fma(omp, Ep - fp, fp));
@@ -802,6 +960,7 @@ __device__ __forceinline__ void relax_cell(Get&& get, Store&& store, const StepP
   };
   Mom<A> m;
   if constexpr (PACKED) m = moments_f2<L, DEV>(get2, (float)c_dev);
+  else if constexpr (std::is_same<A, double>::value) m = moments_fixed<L>(get);
   else m = moments<L, A, DEV>(get, c_dev);
   if constexpr (RELOAD) reload_barrier();
   const Landau<A> lw = landau_step<A>(m, p);
@@ -1412,8 +1571,8 @@ __global__ void __launch_bounds__(kMomThreads) k_fields(const typename S::T* __r
            isfinite(m.Tzz) && isfinite(m.Txy) && isfinite(m.Txz) && isfinite(m.Tyz);
   };
   if constexpr (std::is_same<typename S::A, double>::value) {
-    const Mom<double> m = moments<L, double>([&](auto I) -> double { return src[index(I)]; });
-    put(landau<double, 200>(m));
+    const Mom<double> m = moments_fixed<L>([&](auto I) -> double { return src[index(I)]; });
+    put(landau_f64<200>(m));
     finite = all_finite(m);
     d[0] = m.N0, d[1] = m.T00, d[2] = m.T0x, d[3] = m.T0y, d[4] = m.T0z;
   } else {

@@ -40,7 +40,8 @@ __global__ void __launch_bounds__(kMomThreads) k_densities_noalloc(const typenam
   // cells in double
   double d[5];
   if constexpr (std::is_same<typename S::A, double>::value) {
-    const Mom<double> m = moments<L, double>([&](auto I) -> double { return src[(long long)decltype(I)::value * p.cells + c]; });
+    const Mom<double> m =
+        moments_fixed<L>([&](auto I) -> double { return src[(long long)decltype(I)::value * p.cells + c]; });
     d[0] = m.N0, d[1] = m.T00, d[2] = m.T0x, d[3] = m.T0y, d[4] = m.T0z;
   } else {
     constexpr bool DEV = std::is_same<S, StoreF16Dev>::value;
