@@ -180,6 +180,10 @@ rlb_status rlb_set_populations(rlb_ctx* ctx, const double* f, int on_device);
  *         one warp here instead of two.
  *   19    96-cell row tiles (rows of at most 96 cells; 96, 48 and 32 fill them), four consumer
  *         groups of three warps, one warp per float cell.
+ *   20    the team kernel: the four warps of a block share 32 consecutive cells, a quarter of the
+ *         populations each; every storage and lattice.  On small lattices (the default for those
+ *         whose rows do not suit the pipelined kernel) rlb_step runs up to 64 steps in one
+ *         cooperative launch, with a bounded barrier over the grid after each.
  * Each variant repeats one step from the current populations into the spare buffer `reps` times, so
  * the state does not change; this is allowed only before the first step after rlb_init /
  * rlb_set_populations (RLB_ESTATE otherwise).  *variant (may be NULL) receives the choice;
@@ -202,8 +206,8 @@ rlb_status rlb_autotune(rlb_ctx* ctx, int reps, int* variant, double ms[RLB_MAX_
  * tiles), members that fill a 96-cell row tile better than a 128-cell one through a launch of the
  * 96-cell row-tile kernel with the same warps (variant 19 beside 16), and the other pipelined
  * members through the row-segment kernel of the same block layout.  The others (e.g. 1 x 1 x N
- * tubes) run through the register kernels with the variant a context of that storage runs when it
- * has no pipelined one (3 float, 2 half, 0 double; see rlb_batch_member_variant).  Members keep
+ * tubes) run through the team kernel (float storages; one launch) or, double, the register kernels
+ * (see rlb_batch_member_variant).  Members keep
  * their own buffers, parameters, status and step counters; a member's populations after a batched
  * run are bitwise those of the same steps taken alone with the same step-kernel variant.  Members
  * must use the batch's stream.
@@ -246,7 +250,7 @@ rlb_status rlb_batch_set_variant(rlb_batch* b, int variant);
  * variant: the batch's own; the 96-cell row-tile variant for a member that runs in those beside a
  * 128-cell row-tile variant; for a row-tile variant and a member that runs in row segments, the
  * row-segment variant of the same block layout; for a pipelined variant and a member whose rows do
- * not suit the tiles, the register fallback (3 float, 2 half, 0 double).  Running that member
+ * not suit the tiles, the fallback (20 float storages, 0 double).  Running that member
  * alone with this variant gives the same populations bitwise.  -1 for an empty slot or NULL. */
 int rlb_batch_member_variant(const rlb_batch* b, int slot);
 

@@ -81,6 +81,10 @@ def build(force=False, verbose=False):
         obj = os.path.join(BUILD, "rlb_inst_o%d_s%d.o" % (o, s))
         jobs.append((obj, [nvcc] + NVCC_FLAGS + inc + ["-DRLB_INST_ORDER=%d" % o, "-DRLB_INST_STORAGE=%d" % s,
                                                           "-c", os.path.join(CSRC, "rlb_inst.cu"), "-o", obj]))
+    for o, s in INSTANCES:
+        obj = os.path.join(BUILD, "rlb_inst_o%d_s%d_team.o" % (o, s))
+        jobs.append((obj, [nvcc] + NVCC_FLAGS + inc + ["-DRLB_INST_ORDER=%d" % o, "-DRLB_INST_STORAGE=%d" % s, "-c",
+                                                          os.path.join(CSRC, "rlb_inst_team.cu"), "-o", obj]))
     for o, s, v in VARIANT_UNITS:
         obj = os.path.join(BUILD, "rlb_inst_o%d_s%d_v%d.o" % (o, s, v))
         jobs.append((obj, [nvcc] + NVCC_FLAGS + inc + ["-DRLB_INST_ORDER=%d" % o, "-DRLB_INST_STORAGE=%d" % s,

@@ -139,7 +139,7 @@ extern "C" size_t rlb_bytes_required(const rlb_params* p) {
   const size_t q = p->order == 3 ? Quad3::Q : Quad2::Q;
   const size_t blocks = (cells + kMomThreads - 1) / kMomThreads;
   return 2 * (q * cells * storage_bytes(p->storage) + 2 * kPopGuardBytes) + 6 * cells * sizeof(double) +
-         5 * blocks * sizeof(double) + 5 * sizeof(double) + kStatusWords * sizeof(int);
+         5 * blocks * sizeof(double) + 5 * sizeof(double) + kStatusAlloc * sizeof(int);
 }
 
 template <class L>
@@ -183,7 +183,22 @@ static bool pipe_shape(const rlb_ctx* c, int v, PipeParams* pp, int* grid, int* 
 static bool variant_available(const rlb_ctx* c, int v) {
   if (v < 0) return false;
   if (v < kNumRegVariants) return v < c->launch->step_variants;
+  if (v == kTeamVariant) return true;
   return pipe_shape(c, v, nullptr, nullptr, nullptr, nullptr);
+}
+
+// Lattices the team kernel is for: at most this many tiles per resident block (float storages 4, about
+// 116,000 cells; double 1, 14,600).  Measured per step against the register kernels: 1 x 1 x 2613 float
+// 6.7 us against 33, 32^3 float 17 against 25, 64^3 84 against 87, 151 x 93 x 70 512 against 409;
+// 1 x 1 x 800 double 28 us against 104, 96^3 4.7 ms against 2.3 (there the pipe is busy either way and the
+// team's second and third pass through its code cost more).  They also take several steps per launch: a
+// barrier over the grid is about 1 us, the gap between launches 2 to 4.  64 steps in one launch stay below
+// 20 ms.
+constexpr int kTeamMaxSteps = 64;
+static bool small_for_team(const rlb_ctx* c) {
+  const long long tiles = ((long long)c->cells + kTeamCells - 1) / kTeamCells;
+  const long long room = (long long)c->sms * c->launch->team_resident(c->sp.has_wall);
+  return tiles <= (c->prm.storage == RLB_F64 ? 1 : 4) * room;
 }
 
 // The variant rlb_step uses unless asked otherwise: the first one that suits the context in an
@@ -193,8 +208,8 @@ static bool variant_available(const rlb_ctx* c, int v) {
 // then row segments in three consumer groups; then the register kernels; the register kernel for double storage (whose step is bound by the
 // double-precision pipe, which the register kernel's 4 warps per scheduler keep busier).
 static int default_variant(const rlb_ctx* c) {
-  static const int pref_f32[] = {19, 16, 15, 18, 17, 5, 12, 4, 13, 8, 6, 9, 7, 3};
-  static const int pref_f16[] = {12, 16, 15, 13, 4, 8, 6, 5, 9, 7, 2};
+  static const int pref_f32[] = {19, 16, 15, 18, 17, 5, 12, 4, 13, 8, 6, 9, 7};
+  static const int pref_f16[] = {12, 16, 15, 13, 4, 8, 6, 5, 9, 7};
   const int* pref = c->prm.storage == RLB_F32 ? pref_f32 : pref_f16;
   const int n = c->prm.storage == RLB_F32 ? (int)(sizeof(pref_f32) / sizeof(int)) : (int)(sizeof(pref_f16) / sizeof(int));
   if (c->prm.storage != RLB_F64)
@@ -216,14 +231,20 @@ static int default_variant(const rlb_ctx* c) {
       }
       if (variant_available(c, pref[k])) return pref[k];
     }
-  return kDefaultStepVariant;
+  return small_for_team(c) ? kTeamVariant : (c->prm.storage == RLB_F32 ? 3 : (c->prm.storage == RLB_F16DEV ? 2 : 0));
 }
 
 static rlb_status check_launch(rlb_ctx* c, cudaError_t e, const char* what);
 
+
 // One time step of the whole lattice with step-kernel variant v: the register kernels (two
 // launches: interior rows, then the shell) or the pipelined kernel (one launch).
 static rlb_status launch_step(rlb_ctx* c, int v) {
+  if (v == kTeamVariant)
+    return check_launch(c,
+                        c->launch->team_steps(c->buf[c->cur], c->buf[1 - c->cur], c->sp, c->status, 1, c->sms,
+                                              reinterpret_cast<unsigned*>(c->status + kBarrierWord), c->stream),
+                        "team step kernel");
   if (v >= kNumRegVariants) {
     PipeParams pp;
     int grid = 0, threads = 0, smem = 0, tx = 0, rows = 0, split = 0;
@@ -323,6 +344,7 @@ extern "C" rlb_status rlb_create(const rlb_params* p, rlb_ctx** out) {
   if (e == cudaSuccess) {
     const int want = p->step_variant;
     c->variant = (want >= 0 && variant_available(c, want)) ? want : default_variant(c);
+    c->team_chunk = small_for_team(c) ? kTeamMaxSteps : 1;
   }
   for (int b = 0; b < 2 && e == cudaSuccess; ++b) {
     e = cudaMalloc(&c->raw[b], pop_bytes + 2 * kPopGuardBytes);
@@ -334,7 +356,7 @@ extern "C" rlb_status rlb_create(const rlb_params* p, rlb_ctx** out) {
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->fields, 6 * (size_t)c->cells * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->partial, 5 * (size_t)c->fblocks * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->totals, 5 * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&c->status, kStatusWords * sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&c->status, kStatusAlloc * sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(c->status, 0, kStatusWords * sizeof(int), c->stream);
   if (e != cudaSuccess) {
     const rlb_status st = (e == cudaErrorMemoryAllocation) ? RLB_ENOMEM : RLB_ECUDA;
@@ -498,12 +520,21 @@ extern "C" rlb_status rlb_init(rlb_ctx* c, const double* n, const double* T, con
 extern "C" rlb_status rlb_step(rlb_ctx* c, long nsteps) {
   if (!c) return RLB_EINVAL;
   if (nsteps < 0) return fail(c, RLB_EINVAL, "nsteps < 0");
-  for (long s = 0; s < nsteps; ++s) {
-    rlb_status st = launch_step(c, c->variant);
+  while (nsteps > 0) {
+    const int k = c->variant == kTeamVariant ? (int)std::min<long>(nsteps, c->team_chunk) : 1;
+    rlb_status st = RLB_OK;
+    if (k > 1)
+      st = check_launch(c,
+                        c->launch->team_steps(c->buf[c->cur], c->buf[1 - c->cur], c->sp, c->status, k, c->sms,
+                                              reinterpret_cast<unsigned*>(c->status + kBarrierWord), c->stream),
+                        "team step kernel");
+    else
+      st = launch_step(c, c->variant);
     if (st != RLB_OK) return st;
-    c->cur = 1 - c->cur;
+    c->cur = (c->cur + k) & 1;
     c->have_prev = true;
-    ++c->steps;
+    c->steps += k;
+    nsteps -= k;
   }
   return RLB_OK;
 }

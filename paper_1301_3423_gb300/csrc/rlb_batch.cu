@@ -27,7 +27,7 @@ struct GraphCache {
   cudaGraphExec_t exec = nullptr;
   long nsteps = 0, version = -1;
   int variant = -1, nmembers = 0, tiles = 0, row_tiles = -1, walls = -1, pipe_tiles = -1, pipe_walls = -1,
-      rtile_tiles = -1, r96_tiles = -1;
+      rtile_tiles = -1, r96_tiles = -1, team_tiles = -1;
 };
 
 }  // namespace
@@ -60,6 +60,9 @@ struct rlb_batch {
   int* d_r96_tm = nullptr;       // member index of every 96-cell row tile
   int r96_tm_capacity = 0;
   int r96_tiles = 0;
+  int* d_team_tm = nullptr;      // member index of every team tile
+  int team_tm_capacity = 0;
+  int team_tiles = 0;
   int* pipe_timeout = nullptr;   // status word that counts the pipelined kernel's expired waits
   PipeLayout lay{};              // block layout of the current pipelined variant
   int sms = 0, smem_per_sm = 0, smem_optin = 0;
@@ -113,11 +116,12 @@ static int elem_of(int storage) { return storage == RLB_F64 ? 8 : (storage == RL
 
 // The register-kernel variant for members the pipelined kernel cannot take (rows not on 16-byte
 // boundaries): the one a context of that storage runs when no pipelined variant exists for it.
-static int reg_fallback(const rlb_batch* b) { return b->storage == RLB_F32 ? 3 : (b->storage == RLB_F16DEV ? 2 : 0); }
+static int reg_fallback(const rlb_batch* b) { return b->storage == RLB_F64 ? 0 : kTeamVariant; }
 
 static bool variant_exists(const rlb_batch* b, int v, PipeLayout* lay = nullptr) {
   if (v < 0) return false;
   if (v < kNumRegVariants) return v < b->launch->step_variants;
+  if (v == kTeamVariant) return true;
   const int q = b->order == 3 ? 128 : 66;
   return pipe_layout(v, q, elem_of(b->storage), b->smem_per_sm, b->smem_optin, lay);
 }
@@ -133,7 +137,7 @@ static int row_tile_fill(int nx, int tx) { return nx <= tx ? (tx / nx) * nx : 0;
 // on GB300 at 128^3: one warp per float cell 1.13x faster in row tiles, half storage 1.26x; two
 // warps per float cell 1.04x faster in segments).  96-cell tiles exist as row tiles only.
 static int member_mode(const rlb_batch* b, const StepParams& p, int v, const PipeLayout& lay, const PipeLayout& lay96) {
-  if (v < kNumRegVariants) return 0;
+  if (!is_pipe(v)) return 0;
   const int vmax = b->order == 3 ? Quad3::VMAX_X : Quad2::VMAX_X;
   const int elem = elem_of(b->storage);
   const bool seg = lay.tx != 96 && pipe_fits(p.nx, lay.tx, elem, fill_eighths(lay, elem));
@@ -147,7 +151,7 @@ static int member_mode(const rlb_batch* b, const StepParams& p, int v, const Pip
 
 // The 96-cell row-tile variant with the warps of 128-cell row-tile variant v (-1 if none).
 static int rows96_sibling(int v) {
-  if (v < kNumRegVariants || v >= kNumVariantsTotal) return -1;
+  if (!is_pipe(v)) return -1;
   const PipeConfig& c = kPipeConfigs[v - kNumRegVariants];
   if (!c.rows || c.tx != 128) return -1;
   for (int k = 0; k < kNumPipeConfigs; ++k) {
@@ -162,7 +166,7 @@ static int rows96_sibling(int v) {
 // The row-segment variant with the block layout of row-tile variant v (the shape the batch runs its
 // row-segment members in); v itself if it has no row tiles, -1 if none exists.
 static int segment_sibling(int v) {
-  if (v < kNumRegVariants || v >= kNumVariantsTotal) return v;
+  if (!is_pipe(v)) return v;
   const PipeConfig& c = kPipeConfigs[v - kNumRegVariants];
   if (!c.rows) return v;
   for (int k = 0; k < kNumPipeConfigs; ++k) {
@@ -251,11 +255,12 @@ static rlb_status upload_table(rlb_batch* b, long nsteps, int variant, int* nmem
   b->walls = 0;
   b->pipe_walls = 0;
   b->pipe_timeout = nullptr;
-  const bool pipe = variant >= kNumRegVariants && variant_exists(b, variant, &b->lay);
+  const bool pipe = is_pipe(variant) && variant_exists(b, variant, &b->lay);
+  const bool team = (pipe ? reg_fallback(b) : variant) == kTeamVariant;
   if (!pipe) b->lay = PipeLayout{};
   b->v96 = pipe ? companion96(b, variant, &b->lay96) : -1;
   if (!pipe) b->lay96 = PipeLayout{};
-  std::vector<int> r96_tm;
+  std::vector<int> r96_tm, team_tm;
   for (const Member& m : b->members) {
     if (!m.ctx || m.steps_left <= 0) continue;
     BatchMember d{};
@@ -279,6 +284,12 @@ static rlb_status upload_table(rlb_batch* b, long nsteps, int variant, int* nmem
       continue;
     }
     if (d.p.has_wall) b->walls = 1;
+    if (team) {
+      d.team_tile_begin = (int)team_tm.size();
+      team_tm.resize(team_tm.size() + (d.p.cells + kTeamCells - 1) / kTeamCells, (int)t.size());
+      t.push_back(d);
+      continue;
+    }
     // row tiles: 4 row-kernel warps; shell tiles: 4 shell-row warps (kStepThreads shell cells for
     // members that need the modulo wrap)
     d.row_tile_begin = (int)row_tm.size();
@@ -294,18 +305,21 @@ static rlb_status upload_table(rlb_batch* b, long nsteps, int variant, int* nmem
   b->pipe_tiles = (int)pipe_tm.size();
   b->rtile_tiles = (int)rtile_tm.size();
   b->r96_tiles = (int)r96_tm.size();
+  b->team_tiles = (int)team_tm.size();
   for (BatchMember& d : t) d.shell_tile_begin += b->row_tiles;
   std::vector<int> tm(row_tm);
   tm.insert(tm.end(), shell_tm.begin(), shell_tm.end());
   const int tiles = (int)tm.size();
   *nmembers = (int)t.size();
-  *total_tiles = tiles + b->pipe_tiles + b->rtile_tiles + b->r96_tiles;
+  *total_tiles = tiles + b->pipe_tiles + b->rtile_tiles + b->r96_tiles + b->team_tiles;
   if (t.empty()) return RLB_OK;
   rlb_status st = upload_tiles(b, &b->d_pipe_tm, &b->pipe_tm_capacity, pipe_tm, "pipelined tile table");
   if (st != RLB_OK) return st;
   st = upload_tiles(b, &b->d_rtile_tm, &b->rtile_tm_capacity, rtile_tm, "row-tile table");
   if (st != RLB_OK) return st;
   st = upload_tiles(b, &b->d_r96_tm, &b->r96_tm_capacity, r96_tm, "96-cell row-tile table");
+  if (st != RLB_OK) return st;
+  st = upload_tiles(b, &b->d_team_tm, &b->team_tm_capacity, team_tm, "team tile table");
   if (st != RLB_OK) return st;
   if ((int)t.size() > b->d_capacity) {
     if (b->d_members) cudaFree(b->d_members);
@@ -373,8 +387,13 @@ static rlb_status enqueue_step(rlb_batch* b, int k, int variant, int* counters) 
     ++b->launches;
     if (e != cudaSuccess) return bfail(b, RLB_ECUDA, std::string("batched pipelined step: ") + cudaGetErrorString(e));
   }
+  if (b->team_tiles > 0) {
+    e = b->launch->team_batch_step(b->d_members, b->d_team_tm, b->team_tiles, k, b->walls, b->sms, b->stream);
+    ++b->launches;
+    if (e != cudaSuccess) return bfail(b, RLB_ECUDA, std::string("batched team step: ") + cudaGetErrorString(e));
+  }
   if (b->row_tiles + b->shell_tiles > 0) {
-    const int rv = variant < kNumRegVariants ? variant : reg_fallback(b);
+    const int rv = is_pipe(variant) ? reg_fallback(b) : variant;
     e = b->launch->batch_step(b->d_members, b->d_tile_member, b->row_tiles, b->shell_tiles, k, counters, rv, b->walls,
                               grid_of(b, rv), b->stream);
     b->launches += (b->row_tiles > 0) + (b->shell_tiles > 0);
@@ -417,7 +436,7 @@ extern "C" rlb_status rlb_batch_run(rlb_batch* b, long nsteps, int use_graph, in
       if (!gc.exec || gc.nsteps != nsteps || gc.version != b->version || gc.variant != b->variant ||
           gc.nmembers != nmem || gc.tiles != tiles || gc.row_tiles != b->row_tiles || gc.walls != b->walls ||
           gc.pipe_tiles != b->pipe_tiles || gc.pipe_walls != b->pipe_walls || gc.rtile_tiles != b->rtile_tiles ||
-          gc.r96_tiles != b->r96_tiles) {
+          gc.r96_tiles != b->r96_tiles || gc.team_tiles != b->team_tiles) {
         if (b->graph.exec) cudaGraphExecDestroy(b->graph.exec);
         b->graph.exec = nullptr;
         cudaStream_t cs;
@@ -451,10 +470,11 @@ extern "C" rlb_status rlb_batch_run(rlb_batch* b, long nsteps, int use_graph, in
         gc.pipe_walls = b->pipe_walls;
         gc.rtile_tiles = b->rtile_tiles;
         gc.r96_tiles = b->r96_tiles;
+        gc.team_tiles = b->team_tiles;
       }
       BATCH_CUDA(b, cudaGraphLaunch(b->graph.exec, b->stream));
       b->launches += nsteps * ((b->row_tiles > 0) + (b->shell_tiles > 0) + (b->pipe_tiles > 0) + (b->rtile_tiles > 0) +
-                               (b->r96_tiles > 0));
+                               (b->r96_tiles > 0) + (b->team_tiles > 0));
     } else {
       rlb_status st = enqueue_run(b, nsteps, nmem, tiles, b->variant);
       if (st != RLB_OK) return st;
@@ -532,7 +552,7 @@ extern "C" rlb_status rlb_batch_set_variant(rlb_batch* b, int variant) {
 
 extern "C" int rlb_batch_member_variant(const rlb_batch* b, int slot) {
   if (!b || slot < 0 || slot >= (int)b->members.size() || !b->members[slot].ctx) return -1;
-  if (b->variant < kNumRegVariants) return b->variant;
+  if (!is_pipe(b->variant)) return b->variant;
   PipeLayout lay;
   if (!variant_exists(b, b->variant, &lay)) return reg_fallback(b);
   PipeLayout lay96;
@@ -557,6 +577,7 @@ extern "C" rlb_status rlb_batch_destroy(rlb_batch* b) {
   if (b->d_pipe_tm) cudaFree(b->d_pipe_tm);
   if (b->d_rtile_tm) cudaFree(b->d_rtile_tm);
   if (b->d_r96_tm) cudaFree(b->d_r96_tm);
+  if (b->d_team_tm) cudaFree(b->d_team_tm);
   if (b->d_counters) cudaFree(b->d_counters);
   delete b;
   return RLB_OK;

@@ -34,7 +34,16 @@ constexpr PipeConfig kPipeConfigs[] = {
     {128, 8, 1, 4, 1, 1}, {128, 8, 1, 8, 1, 1},  {128, 4, 1, 4, 1, 1}, {128, 12, 1, 4, 0, 0},
     {128, 12, 1, 4, 1, 0}, {128, 12, 1, 2, 0, 0}, {128, 12, 1, 2, 1, 0}, {96, 12, 1, 4, 1, 0}};
 constexpr int kNumPipeConfigs = sizeof(kPipeConfigs) / sizeof(kPipeConfigs[0]);
-constexpr int kNumVariantsTotal = kNumRegVariants + kNumPipeConfigs;
+// Variant after the pipelined shapes: the team kernel (rlb_team.cuh), for every storage and lattice.
+constexpr int kTeamVariant = kNumRegVariants + kNumPipeConfigs;
+constexpr int kNumVariantsTotal = kTeamVariant + 1;
+constexpr bool is_pipe(int v) { return v >= kNumRegVariants && v < kTeamVariant; }
+constexpr int kTeamWarps = 4;   // warps that share a cell
+constexpr int kTeamCells = 32;  // cells per tile
+// Resident blocks per SM the team kernels' registers are cut to: 6 x 4 warps for float (80 registers),
+// 3 for double (a quarter of the populations is 64 registers).
+template <class A>
+constexpr int kTeamBlocks = sizeof(A) == 8 ? 3 : 6;
 constexpr int kPipeMaxStages = 16;
 constexpr int kPipeMaxConsumerWarps = 12;
 constexpr int kPipeMaxProducerWarps = 12;
@@ -91,6 +100,8 @@ enum : int {
   kStatusBounds = 4,
   kStatusWords = 8
 };
+// Ints allocated with the status words after them: a cache line for the team kernel's grid barrier.
+constexpr int kBarrierWord = 32, kStatusAlloc = 64;
 
 // StepParams::debug bits (testing only)
 enum : int { kDebugStallProducers = 1 };  // the pipelined step's producers do nothing: every wait runs out
@@ -121,6 +132,7 @@ struct BatchMember {
   int row_tile_begin;    // first of its row tiles (4 row-kernel warps each) in the row queue
   int shell_tile_begin;  // first of its shell tiles (kStepThreads shell cells each) in the shell queue
   int pipe_tile_begin;   // first of its tiles in the pipelined kernel's tile list (k_step_pipe_batch)
+  int team_tile_begin;   // first of its tiles in the team kernel's tile list (k_step_team_batch)
 };
 
 }  // namespace rlb

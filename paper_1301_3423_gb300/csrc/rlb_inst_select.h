@@ -65,6 +65,14 @@ RLB_DECLARE_ROWS(128)
 RLB_DECLARE_ROWS(96)
 #undef RLB_DECLARE_ROWS
 
+// Team kernels (rlb_inst_team.cu).
+#define RLB_TFN(fn) RLB_CAT7(team_, fn, _o, RLB_INST_ORDER, _s, RLB_INST_STORAGE, )
+cudaError_t RLB_TFN(steps)(void* a, void* b, const StepParams& p, int* status, int nsteps, int sms, unsigned* arrived,
+                           cudaStream_t s);
+int RLB_TFN(resident)(int walls);
+cudaError_t RLB_TFN(batch)(const BatchMember* m, const int* tm, int ntiles, int launch, int walls, int sms,
+                           cudaStream_t s);
+
 RLB_DECLARE_VARIANT(0)
 RLB_DECLARE_VARIANT(1)
 RLB_DECLARE_VARIANT(2)

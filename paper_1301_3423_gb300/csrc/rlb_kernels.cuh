@@ -355,104 +355,136 @@ __device__ __forceinline__ Mom<A> moments(Get&& get, A c = A(0)) {
   return m;
 }
 
-// The mirror pairs of each energy level, in order.
+// Double arithmetic handles the mirror pairs in four slices: pairs in order of their energy level, a
+// quarter each.  A slice's integer sums (below) have their own grid per level, so the slices define
+// the rounding, and every double kernel, whether one thread or four share a cell, adds the same four.
 template <class L>
-struct LevelPairs {
-  __host__ __device__ static constexpr int count(int l) {
+struct Slices {
+  static constexpr int N = 4, PAIRS = L::Q / 2, PER = (PAIRS + N - 1) / N;
+  __host__ __device__ static constexpr int slice_of(int pair) {
+    int r = 0;  // the pair's rank by (level, index)
+    for (int k = 0; k < PAIRS; ++k)
+      r += L::LEV[2 * k] < L::LEV[2 * pair] || (L::LEV[2 * k] == L::LEV[2 * pair] && k < pair);
+    return r / PER;
+  }
+  // pairs of slice s (of level l if l >= 0), and the + population of the j-th of them
+  __host__ __device__ static constexpr int count(int s, int l = -1) {
     int n = 0;
-    for (int i = 0; i < L::Q; i += 2) n += L::LEV[i] == l;
+    for (int k = 0; k < PAIRS; ++k) n += slice_of(k) == s && (l < 0 || L::LEV[2 * k] == l);
     return n;
   }
-  __host__ __device__ static constexpr int first(int l, int j) {  // the + population of pair j
-    for (int i = 0; i < L::Q; i += 2)
-      if (L::LEV[i] == l && j-- == 0) return i;
+  __host__ __device__ static constexpr int pair(int s, int l, int j) {
+    for (int k = 0; k < PAIRS; ++k)
+      if (slice_of(k) == s && (l < 0 || L::LEV[2 * k] == l) && j-- == 0) return 2 * k;
     return -1;
   }
-  __host__ __device__ static constexpr int sum(int l, int a, int b) {  // of v_a v_b over the pairs
-    int s = 0;
-    for (int i = 0; i < L::Q; i += 2) {
-      const int v[3] = {L::VX[i], L::VY[i], L::VZ[i]};
-      if (L::LEV[i] == l) s += v[a] * v[b];
+  __host__ __device__ static constexpr int sum(int s, int l, int a, int b) {  // of v_a v_b
+    int r = 0;
+    for (int k = 0; k < PAIRS; ++k) {
+      const int v[3] = {L::VX[2 * k], L::VY[2 * k], L::VZ[2 * k]};
+      if (slice_of(k) == s && L::LEV[2 * k] == l) r += v[a] * v[b];
     }
-    return s;
+    return r;
   }
 };
 
-// Moments of double populations, summed in 64-bit integers.  GB300's double pipe retires 2 lanes a
-// clock and SM and bounds the double step; its integer pipe is some 30 times wider.  Per energy level
-// the populations are put on a common grid of 2^-50 to 2^-51 of the level's largest (adding
-// 1.5 2^k leaves the grid value in the low bits of the sum), and the level's sums over v with the
-// integer weights 1, v_a, v_a v_b are exact integers: |v_a v_b| sums to at most 2^11 over the
-// populations, so 51 + 11 bits and the sign fit.  Per level 9 sums return to double and take p0 and
-// p0^2.  The grid is per level, so the rare high levels, which p0^2 weights most, are rounded by their
-// own size: the moments' error is below that of adding the 128 terms in double.  Double operations a
-// cell: 128 adds and 36 conversions, 115 more; 960 when the sums were double.  Integer sums do not
-// depend on their order, so every kernel gets the same bits.
+// Moments of double populations, summed in 64-bit integers.  GB300's double pipe takes 19 clocks an
+// SM for a warp instruction (measured; 64 for a lone warp) and bounds the double step; its integer
+// pipe is some 40 times wider.  Per slice and energy level the populations are put on a common grid
+// of 2^-50 to 2^-51 of the largest of them (adding 1.5 2^k leaves the grid value in the low bits of
+// the sum), and the sums over v with the integer weights 1, v_a, v_a v_b are exact integers:
+// |v_a v_b| sums to at most 2^11 over the populations, so 51 + 11 bits and the sign fit.  Then 9 sums
+// return to double and take p0 and p0^2.  The grid is per level, so the rare high levels, which p0^2
+// weights most, are rounded by their own size: the moments' error is below that of adding the 128
+// terms in double (fields of a 96^3 run against 64-bit references: 4.2e-16 here, 4.6e-16 before).
+// Double operations a cell: 128 adds, 63 conversions, 140 more; 960 when the sums were double.
 // Populations that are not finite (or beyond 2^1021, whose moments overflow) give NaN moments.
-template <class L, class Get>
-__device__ __forceinline__ Mom<double> moments_fixed(Get&& get) {
+// Slice SL's part, before the factors 1 / R and 1 / R^2 (finish_fixed).
+template <class L, int SL, class Get>
+__device__ __forceinline__ Mom<double> moments_fixed_slice(Get&& get) {
   using u64 = unsigned long long;
+  using G = Slices<L>;
   Mom<double> m;
   m.N0 = m.Nx = m.Ny = m.Nz = 0.0;
   m.T00 = m.T0x = m.T0y = m.T0z = 0.0;
-  m.Txx = m.Tyy = m.Txy = m.Txz = m.Tyz = 0.0;
+  m.Txx = m.Tyy = m.Tzz = m.Txy = m.Txz = m.Tyz = 0.0;
   bool finite = true;
   static_for<L::NLEV>([&](auto K) {
     constexpr int l = decltype(K)::value;
-    constexpr int n = LevelPairs<L>::count(l);
-    double f[2 * n];
-    unsigned top = 0;
-    static_for<n>([&](auto J) {
-      constexpr int j = decltype(J)::value, i = LevelPairs<L>::first(l, j);
-      f[2 * j] = get(ic<i>{});
-      f[2 * j + 1] = get(ic<i + 1>{});
-      top = max(top, max((unsigned)__double2hiint(f[2 * j]) & 0x7fffffffu,
-                         (unsigned)__double2hiint(f[2 * j + 1]) & 0x7fffffffu));
-    });
-    const int e = max((int)(top >> 20), 64);  // |f| < 2^(e - 1022)
-    finite = finite && e < 2045;
-    const double C = __hiloint2double(((e + 2) << 20) | 0x80000, 0);  // 1.5 2^(e - 1021)
-    const u64 Cb = (u64)__double_as_longlong(C);
-    // sums of the raw bits; each carries a known multiple of those of C, removed below (modulo 2^64)
-    u64 s0 = 0, sxx = 0, syy = 0, sxy = 0, sxz = 0, syz = 0, sx = 0, sy = 0, sz = 0;
-    static_for<n>([&](auto J) {
-      constexpr int j = decltype(J)::value, i = LevelPairs<L>::first(l, j);
-      constexpr int vx = L::VX[i], vy = L::VY[i], vz = L::VZ[i];
-      const u64 a = (u64)__double_as_longlong(__dadd_rn(f[2 * j], C));
-      const u64 b = (u64)__double_as_longlong(__dadd_rn(f[2 * j + 1], C));
-      const u64 sp = a + b, sm = a - b;
-      s0 += sp;
-      if constexpr (vx != 0) sxx += (u64)(long long)(vx * vx) * sp, sx += (u64)(long long)vx * sm;
-      if constexpr (vy != 0) syy += (u64)(long long)(vy * vy) * sp, sy += (u64)(long long)vy * sm;
-      if constexpr (vz != 0) sz += (u64)(long long)vz * sm;
-      if constexpr (vx * vy != 0) sxy += (u64)(long long)(vx * vy) * sp;
-      if constexpr (vx * vz != 0) sxz += (u64)(long long)(vx * vz) * sp;
-      if constexpr (vy * vz != 0) syz += (u64)(long long)(vy * vz) * sp;
-    });
-    auto even = [&](u64 s, int w) { return (double)(long long)(s - (u64)(2ll * w) * Cb); };
-    const double g = __hiloint2double((e - 50) << 20, 0);  // the grid, 2^(e - 1073)
-    const double p1 = L::P0[l] * g, p2 = L::P0[l] * L::P0[l] * g;
-    const double d0 = even(s0, n), dx = (double)(long long)sx, dy = (double)(long long)sy, dz = (double)(long long)sz;
-    m.N0 = fma(p1, d0, m.N0);
-    m.Nx = fma(p1, dx, m.Nx);
-    m.Ny = fma(p1, dy, m.Ny);
-    m.Nz = fma(p1, dz, m.Nz);
-    m.T00 = fma(p2, d0, m.T00);
-    m.T0x = fma(p2, dx, m.T0x);
-    m.T0y = fma(p2, dy, m.T0y);
-    m.T0z = fma(p2, dz, m.T0z);
-    m.Txx = fma(p2, even(sxx, ic<LevelPairs<L>::sum(l, 0, 0)>::value), m.Txx);
-    m.Tyy = fma(p2, even(syy, ic<LevelPairs<L>::sum(l, 1, 1)>::value), m.Tyy);
-    m.Txy = fma(p2, even(sxy, ic<LevelPairs<L>::sum(l, 0, 1)>::value), m.Txy);
-    m.Txz = fma(p2, even(sxz, ic<LevelPairs<L>::sum(l, 0, 2)>::value), m.Txz);
-    m.Tyz = fma(p2, even(syz, ic<LevelPairs<L>::sum(l, 1, 2)>::value), m.Tyz);
+    constexpr int n = G::count(SL, l);
+    if constexpr (n > 0) {
+      double f[2 * n];
+      unsigned top = 0;
+      static_for<n>([&](auto J) {
+        constexpr int j = decltype(J)::value, i = G::pair(SL, l, j);
+        f[2 * j] = get(ic<i>{});
+        f[2 * j + 1] = get(ic<i + 1>{});
+        top = max(top, max((unsigned)__double2hiint(f[2 * j]) & 0x7fffffffu,
+                           (unsigned)__double2hiint(f[2 * j + 1]) & 0x7fffffffu));
+      });
+      const int e = max((int)(top >> 20), 64);  // |f| < 2^(e - 1022)
+      finite = finite && e < 2045;
+      const double C = __hiloint2double(((e + 2) << 20) | 0x80000, 0);  // 1.5 2^(e - 1021)
+      const u64 Cb = (u64)__double_as_longlong(C);
+      // sums of the raw bits; each carries a known multiple of those of C, removed below (modulo 2^64)
+      u64 s0 = 0, sxx = 0, syy = 0, sxy = 0, sxz = 0, syz = 0, sx = 0, sy = 0, sz = 0;
+      static_for<n>([&](auto J) {
+        constexpr int j = decltype(J)::value, i = G::pair(SL, l, j);
+        constexpr int vx = L::VX[i], vy = L::VY[i], vz = L::VZ[i];
+        const u64 a = (u64)__double_as_longlong(__dadd_rn(f[2 * j], C));
+        const u64 b = (u64)__double_as_longlong(__dadd_rn(f[2 * j + 1], C));
+        const u64 sp = a + b, sm = a - b;
+        s0 += sp;
+        if constexpr (vx != 0) sxx += (u64)(long long)(vx * vx) * sp, sx += (u64)(long long)vx * sm;
+        if constexpr (vy != 0) syy += (u64)(long long)(vy * vy) * sp, sy += (u64)(long long)vy * sm;
+        if constexpr (vz != 0) sz += (u64)(long long)vz * sm;
+        if constexpr (vx * vy != 0) sxy += (u64)(long long)(vx * vy) * sp;
+        if constexpr (vx * vz != 0) sxz += (u64)(long long)(vx * vz) * sp;
+        if constexpr (vy * vz != 0) syz += (u64)(long long)(vy * vz) * sp;
+      });
+      auto even = [&](u64 s, int w) { return (double)(long long)(s - (u64)(2ll * w) * Cb); };
+      const double g = __hiloint2double((e - 50) << 20, 0);  // the grid, 2^(e - 1073)
+      const double p1 = L::P0[l] * g, p2 = L::P0[l] * L::P0[l] * g;
+      const double d0 = even(s0, n), dx = (double)(long long)sx, dy = (double)(long long)sy, dz = (double)(long long)sz;
+      m.N0 = fma(p1, d0, m.N0);
+      m.Nx = fma(p1, dx, m.Nx);
+      m.Ny = fma(p1, dy, m.Ny);
+      m.Nz = fma(p1, dz, m.Nz);
+      m.T00 = fma(p2, d0, m.T00);
+      m.T0x = fma(p2, dx, m.T0x);
+      m.T0y = fma(p2, dy, m.T0y);
+      m.T0z = fma(p2, dz, m.T0z);
+      m.Txx = fma(p2, even(sxx, ic<G::sum(SL, l, 0, 0)>::value), m.Txx);
+      m.Tyy = fma(p2, even(syy, ic<G::sum(SL, l, 1, 1)>::value), m.Tyy);
+      m.Txy = fma(p2, even(sxy, ic<G::sum(SL, l, 0, 1)>::value), m.Txy);
+      m.Txz = fma(p2, even(sxz, ic<G::sum(SL, l, 0, 2)>::value), m.Txz);
+      m.Tyz = fma(p2, even(syz, ic<G::sum(SL, l, 1, 2)>::value), m.Tyz);
+    }
   });
+  if (!finite) m.N0 = m.T00 = __longlong_as_double(0x7ff8000000000000ll);
+  return m;
+}
+__device__ __forceinline__ void add_moments(Mom<double>& m, const Mom<double>& a) {
+  m.N0 = __dadd_rn(m.N0, a.N0), m.Nx = __dadd_rn(m.Nx, a.Nx), m.Ny = __dadd_rn(m.Ny, a.Ny);
+  m.Nz = __dadd_rn(m.Nz, a.Nz), m.T00 = __dadd_rn(m.T00, a.T00), m.T0x = __dadd_rn(m.T0x, a.T0x);
+  m.T0y = __dadd_rn(m.T0y, a.T0y), m.T0z = __dadd_rn(m.T0z, a.T0z), m.Txx = __dadd_rn(m.Txx, a.Txx);
+  m.Tyy = __dadd_rn(m.Tyy, a.Tyy), m.Txy = __dadd_rn(m.Txy, a.Txy), m.Txz = __dadd_rn(m.Txz, a.Txz);
+  m.Tyz = __dadd_rn(m.Tyz, a.Tyz);
+}
+template <class L>
+__device__ __forceinline__ void finish_fixed(Mom<double>& m) {
   m.Nx *= L::INV_R, m.Ny *= L::INV_R, m.Nz *= L::INV_R;
   m.T0x *= L::INV_R, m.T0y *= L::INV_R, m.T0z *= L::INV_R;
-  m.Txx *= L::INV_R2, m.Tyy *= L::INV_R2, m.Txy *= L::INV_R2, m.Txz *= L::INV_R2, m.Tyz *= L::INV_R2;
-  if (!finite) m.N0 = m.T00 = __longlong_as_double(0x7ff8000000000000ll);
+  m.Txx = __dmul_rn(m.Txx, L::INV_R2), m.Tyy = __dmul_rn(m.Tyy, L::INV_R2);
+  m.Txy *= L::INV_R2, m.Txz *= L::INV_R2, m.Tyz *= L::INV_R2;
   // |v|^2 = R^2 for every velocity, so the spatial trace of T equals T^00.
   m.Tzz = m.T00 - m.Txx - m.Tyy;
+}
+template <class L, class Get>
+__device__ __forceinline__ Mom<double> moments_fixed(Get&& get) {
+  Mom<double> m = moments_fixed_slice<L, 0>(get);
+  static_for<Slices<L>::N - 1>([&](auto K) { add_moments(m, moments_fixed_slice<L, decltype(K)::value + 1>(get)); });
+  finish_fixed<L>(m);
   return m;
 }
 
@@ -752,6 +784,39 @@ __device__ __forceinline__ LevCoef<L, A> level_coef(const EqCoef<L::ORDER, A>& q
 //   f*_i = f_i + omega_i (w_i E_i - f_i),  omega_i = p_i.U / (tau' p0_i) = (U0 - t_i) / tau'.
 // DEV = true: get / put carry deviations d_i = f_i / w_i - c, and the collision is
 // d_i + omega_i ((E_i - c) - d_i).
+// The part of it that +v (population I) and -v share: t = v.U / R of +v and the two omegas.
+template <class A>
+struct DirTerm {
+  A t, t2, omp, omm;
+};
+template <class L, class A, int I>
+__device__ __forceinline__ DirTerm<A> dir_term(A Ux, A Uy, A Uz, A inv_tau, A a) {
+  constexpr int vx = L::VX[I], vy = L::VY[I], vz = L::VZ[I];
+  constexpr double ir = L::INV_R;
+  A t = A(0);  // direction +v: t; mirror -v: -t
+  if constexpr (vx != 0) t = fma(A(vx * ir), Ux, t);
+  if constexpr (vy != 0) t = fma(A(vy * ir), Uy, t);
+  if constexpr (vz != 0) t = fma(A(vz * ir), Uz, t);
+  return DirTerm<A>{t, t * t, fma(-t, inv_tau, a), fma(t, inv_tau, a)};
+}
+// One mirror pair.  The even part a + c t^2 and the odd part's factor b + d t^2 serve both signs of t.
+template <class L, class A, bool DEV, int IP, class Get, class Put>
+__device__ __forceinline__ void collide_pair(const DirTerm<A>& k, A ea, A eb, A ec, A ed, Get&& get, Put&& put) {
+  const A w = A(L::W[IP]);
+  const A even = fma(k.t2, ec, ea);
+  A odd = eb;
+  if constexpr (L::ORDER == 3) odd = fma(k.t2, ed, odd);
+  const A Ep = fma(k.t, odd, even), Em = fma(-k.t, odd, even);
+  const A fp = get(ic<IP>{}), fm = get(ic<IP + 1>{});
+  if constexpr (DEV) {
+    put(ic<IP>{}, fma(k.omp, Ep - fp, fp));
+    put(ic<IP + 1>{}, fma(k.omm, Em - fm, fm));
+    (void)w;
+  } else {
+    put(ic<IP>{}, fma(k.omp, fma(w, Ep, -fp), fp));
+    put(ic<IP + 1>{}, fma(k.omm, fma(w, Em, -fm), fm));
+  }
+}
 template <class L, class A, bool DEV = false, class Get, class Put>
 __device__ __forceinline__ void collide(const Landau<A>& lw, A T, A inv_tau, Get&& get, Put&& put, A c = A(0)) {
   const LevCoef<L, A> e = level_coef<L, A>(eq_coef<L::ORDER, A>(lw.n, T, lw.U0), DEV ? c : A(0));
@@ -759,34 +824,11 @@ __device__ __forceinline__ void collide(const Landau<A>& lw, A T, A inv_tau, Get
   static_for<L::NDP>([&](auto K) {
     constexpr int k = decltype(K)::value;
     constexpr int first = L::DP_FIRST[k];
-    constexpr int np = L::DP_NPAIR[k];
-    constexpr int vx = L::VX[first], vy = L::VY[first], vz = L::VZ[first];
-    constexpr double ir = L::INV_R;
-    A t = A(0);  // direction +v: t; mirror -v: -t
-    if constexpr (vx != 0) t = fma(A(vx * ir), lw.Ux, t);
-    if constexpr (vy != 0) t = fma(A(vy * ir), lw.Uy, t);
-    if constexpr (vz != 0) t = fma(A(vz * ir), lw.Uz, t);
-    const A t2 = t * t;
-    const A omp = fma(-t, inv_tau, a), omm = fma(t, inv_tau, a);
-    static_for<np>([&](auto J) {
+    const DirTerm<A> dt = dir_term<L, A, first>(lw.Ux, lw.Uy, lw.Uz, inv_tau, a);
+    static_for<L::DP_NPAIR[k]>([&](auto J) {
       constexpr int ip = first + 2 * decltype(J)::value;
       constexpr int l = L::LEV[ip];
-      constexpr double wd = L::W[ip];
-      const A w = A(wd);
-      // the even part a + c t^2 and the odd part's factor b + d t^2 serve both signs of t
-      const A even = fma(t2, e.c[l], e.a[l]);
-      A odd = e.b[l];
-      if constexpr (L::ORDER == 3) odd = fma(t2, e.d[l], odd);
-      const A Ep = fma(t, odd, even), Em = fma(-t, odd, even);
-      const A fp = get(ic<ip>{}), fm = get(ic<ip + 1>{});
-      if constexpr (DEV) {
-        put(ic<ip>{}, fma(omp, Ep - fp, fp));
-        put(ic<ip + 1>{}, fma(omm, Em - fm, fm));
-        (void)w;
-      } else {
-        put(ic<ip>{}, fma(omp, fma(w, Ep, -fp), fp));
-        put(ic<ip + 1>{}, fma(omm, fma(w, Em, -fm), fm));
-      }
+      collide_pair<L, A, DEV, ip>(dt, e.a[l], e.b[l], e.c[l], e.d[l], get, put);
     });
   });
 }
@@ -889,25 +931,34 @@ __device__ __forceinline__ Mom<float> moments_f2(Get2&& get2, float c = 0.f) {
   return m;
 }
 
+// What the paired collision of one cell needs: the level coefficients, U and the relaxation rate.
+template <class L>
+struct CollideCoef {
+  LevCoef<L, float> e;
+  float Ux, Uy, Uz, inv_tau, a;  // a = U0 / tau'
+};
+template <class L, bool DEV>
+__device__ __forceinline__ CollideCoef<L> collide_coef(const Landau<float>& lw, float T, float inv_tau, float c) {
+  return CollideCoef<L>{level_coef<L, float>(eq_coef<L::ORDER, float>(lw.n, T, lw.U0), DEV ? c : 0.f), lw.Ux, lw.Uy,
+                        lw.Uz, inv_tau, lw.U0 * inv_tau};
+}
+
 // Collision of the direction pairs [DPB, DPE) (all of them by default).
 template <class L, bool DEV = false, int DPB = 0, int DPE = L::NDP, class Get2, class Put2>
-__device__ __forceinline__ void collide_f2(const Landau<float>& lw, float T, float inv_tau, Get2&& get2, Put2&& put2,
-                                           float c = 0.f) {
-  const LevCoef<L, float> e1 = level_coef<L, float>(eq_coef<L::ORDER, float>(lw.n, T, lw.U0), DEV ? c : 0.f);
+__device__ __forceinline__ void collide_f2(const CollideCoef<L>& q, Get2&& get2, Put2&& put2) {
   // the coefficients as (x, x) pairs once per cell, the operands of the paired Horner steps
   struct {
     float2 a[L::NLEV], b[L::NLEV], c[L::NLEV], d[L::NLEV];
   } e;
   static_for<L::NLEV>([&](auto K) {
     constexpr int l = decltype(K)::value;
-    e.a[l] = f2(e1.a[l], e1.a[l]);
-    e.b[l] = f2(e1.b[l], e1.b[l]);
-    e.c[l] = f2(e1.c[l], e1.c[l]);
-    e.d[l] = f2(e1.d[l], e1.d[l]);
+    e.a[l] = f2(q.e.a[l], q.e.a[l]);
+    e.b[l] = f2(q.e.b[l], q.e.b[l]);
+    e.c[l] = f2(q.e.c[l], q.e.c[l]);
+    e.d[l] = f2(q.e.d[l], q.e.d[l]);
   });
-  const float a = lw.U0 * inv_tau;
-  const float2 Uxp = f2(lw.Ux, lw.Ux), Uyp = f2(lw.Uy, lw.Uy), Uzp = f2(lw.Uz, lw.Uz);
-  const float2 itp = f2(inv_tau, inv_tau), nap = f2(-a, -a);
+  const float2 Uxp = f2(q.Ux, q.Ux), Uyp = f2(q.Uy, q.Uy), Uzp = f2(q.Uz, q.Uz);
+  const float2 itp = f2(q.inv_tau, q.inv_tau), nap = f2(-q.a, -q.a);
   static_for<DPE - DPB>([&](auto K) {
     constexpr int k = DPB + decltype(K)::value;
     constexpr int first = L::DP_FIRST[k];
@@ -980,7 +1031,7 @@ __device__ __forceinline__ void relax_cell(Get&& get, Store&& store, const StepP
       store(ic<i>{}, v.x);
       store(ic<i + 1>{}, v.y);
     };
-    collide_f2<L, DEV>(lw, T, inv_tau, get2, put2, (float)c_dev);
+    collide_f2<L, DEV>(collide_coef<L, DEV>(lw, T, inv_tau, (float)c_dev), get2, put2);
   } else {
     collide<L, A, DEV>(lw, T, inv_tau, get, store, c_dev);
   }

@@ -33,6 +33,15 @@ struct Launchers {
   // (tx 128 or 96), float cells split between two warps if split != 0 (float storage)
   cudaError_t (*pipe_step)(const void* src, void* dst, const StepParams& p, const PipeParams& pp, int* status, int tx,
                            int rows, int split, int grid, int threads, int smem, cudaStream_t s);
+  // nsteps time steps of the team kernel from buffer a into buffer b and back (one launch; more than
+  // one step is a cooperative launch whose blocks wait for each other, counted in *arrived)
+  cudaError_t (*team_steps)(void* a, void* b, const StepParams& p, int* status, int nsteps, int sms, unsigned* arrived,
+                            cudaStream_t s);
+  // blocks per SM of that launch
+  int (*team_resident)(int walls);
+  // one time step (launch index `launch`) of the batch members' team tiles
+  cudaError_t (*team_batch_step)(const BatchMember* members, const int* tile_member, int ntiles, int launch, int walls,
+                                 int sms, cudaStream_t s);
   // one time step of the batched pipelined kernel (launch index `launch`) over the members' tiles;
   // walls != 0 selects the kernel with the bounce-back patch
   cudaError_t (*pipe_batch_step)(const BatchMember* members, const int* tile_member, int launch, const PipeParams& pp,
@@ -95,7 +104,7 @@ inline long long pipe_tile_count(int nx, int ny, int nz, int tx, int rows) {
 }
 
 inline bool pipe_layout(int v, int q, int elem, int smem_per_sm, int smem_optin, PipeLayout* out) {
-  if (v < kNumRegVariants || v >= kNumVariantsTotal) return false;
+  if (!is_pipe(v)) return false;
   const PipeConfig& cf = kPipeConfigs[v - kNumRegVariants];
   const int A = 16 / elem;
   const long long stage = (long long)q * (cf.tx + A) * elem;

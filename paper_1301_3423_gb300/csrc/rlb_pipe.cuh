@@ -525,8 +525,9 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
           store(ic<i>{}, v.x);
           store(ic<i + 1>{}, v.y);
         };
-        if (half == 0) collide_f2<L, DEV, 0, KS>(lw, Tl, inv_tau, get2, put2, c_dev);
-        else collide_f2<L, DEV, KS, L::NDP>(lw, Tl, inv_tau, get2, put2, c_dev);
+        const CollideCoef<L> q = collide_coef<L, DEV>(lw, Tl, inv_tau, c_dev);
+        if (half == 0) collide_f2<L, DEV, 0, KS>(q, get2, put2);
+        else collide_f2<L, DEV, KS, L::NDP>(q, get2, put2);
       }
     }
     __syncwarp();
