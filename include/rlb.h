@@ -183,7 +183,8 @@ rlb_status rlb_set_populations(rlb_ctx* ctx, const double* f, int on_device);
  *   20    the team kernel: the four warps of a block share 32 consecutive cells, a quarter of the
  *         populations each; every storage and lattice.  On small lattices (the default for those
  *         whose rows do not suit the pipelined kernel) rlb_step runs up to 64 steps in one
- *         cooperative launch, with a bounded barrier over the grid after each.
+ *         cooperative launch, with a bounded barrier over the grid after each; one launch per step
+ *         when step_variant asked for it.
  * Each variant repeats one step from the current populations into the spare buffer `reps` times, so
  * the state does not change; this is allowed only before the first step after rlb_init /
  * rlb_set_populations (RLB_ESTATE otherwise).  *variant (may be NULL) receives the choice;

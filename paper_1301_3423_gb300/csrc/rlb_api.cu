@@ -344,7 +344,8 @@ extern "C" rlb_status rlb_create(const rlb_params* p, rlb_ctx** out) {
   if (e == cudaSuccess) {
     const int want = p->step_variant;
     c->variant = (want >= 0 && variant_available(c, want)) ? want : default_variant(c);
-    c->team_chunk = small_for_team(c) ? kTeamMaxSteps : 1;
+    // a variant that was asked for takes one launch per step, as the autotuner times it
+    c->team_chunk = want != kTeamVariant && small_for_team(c) ? kTeamMaxSteps : 1;
   }
   for (int b = 0; b < 2 && e == cudaSuccess; ++b) {
     e = cudaMalloc(&c->raw[b], pop_bytes + 2 * kPopGuardBytes);
