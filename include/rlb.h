@@ -176,8 +176,8 @@ rlb_status rlb_set_populations(rlb_ctx* ctx, const double* f, int on_device);
  *         only for lattices with a periodic x of at most 128 cells (and at least the stencil's
  *         x reach), nx again a multiple of 16 bytes' worth of populations.
  *   15..18 row segments (15, 17) and row tiles (16, 18) in three consumer groups of four warps
- *         per block, 4 (15, 16) or 2 (17, 18) producer warps; float storage relaxes each cell in
- *         one warp here instead of two.
+ *         per block, 8 (15, 16) or 2 (17, 18) producer warps; float storage relaxes each cell in
+ *         one warp here instead of two, and row segments are refilled in four chunks.
  *   19    96-cell row tiles (rows of at most 96 cells; 96, 48 and 32 fill them), four consumer
  *         groups of three warps, one warp per float cell.
  *   20    the team kernel: the four warps of a block share 32 consecutive cells, a quarter of the
@@ -185,6 +185,9 @@ rlb_status rlb_set_populations(rlb_ctx* ctx, const double* f, int on_device);
  *         whose rows do not suit the pipelined kernel) rlb_step runs up to 64 steps in one
  *         cooperative launch, with a bounded barrier over the grid after each; one launch per step
  *         when step_variant asked for it.
+ *   21..23 row tiles of 160, 192 and 256 cells (periodic x of at most that many cells), two consumer
+ *         groups, one warp per float cell; float storages, 256 only for half storage and the second
+ *         order.
  * Each variant repeats one step from the current populations into the spare buffer `reps` times, so
  * the state does not change; this is allowed only before the first step after rlb_init /
  * rlb_set_populations (RLB_ESTATE otherwise).  *variant (may be NULL) receives the choice;

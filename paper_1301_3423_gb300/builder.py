@@ -26,6 +26,9 @@ INSTANCES = [(o, s) for o in (3, 2) for s in (0, 1, 2)]
 VARIANT_UNITS = [(o, s, v) for o, s in INSTANCES for v in ((0,) if s == 0 else (0, 1, 2, 3))]
 # pipelined step kernel per (order, storage), tile width and tile kind (row tiles: widths 128 and 96)
 PIPE_UNITS = [(o, s, tx, rows) for o, s in INSTANCES for tx, rows in ((64, 0), (128, 0), (128, 1), (96, 1))]
+# the wide row tiles: float storages, 256 cells where two stages fit
+PIPE_UNITS += [(o, s, tx, 1) for o, s in INSTANCES for tx in (160, 192, 256)
+               if s > 0 and (tx < 256 or s == 2 or o == 2)]
 
 
 def _nvcc():

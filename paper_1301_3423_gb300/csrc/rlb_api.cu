@@ -201,36 +201,47 @@ static bool small_for_team(const rlb_ctx* c) {
   return tiles <= (c->prm.storage == RLB_F64 ? 1 : 4) * room;
 }
 
-// The variant rlb_step uses unless asked otherwise: the first one that suits the context in an
-// order measured on GB300 (32^3 to 256^3 lattices, third order): for float storage one warp per
-// cell in 96-cell row tiles where the rows fill them exactly, then in 128-cell row tiles, then in
-// row segments (0.83 of the copy bandwidth at 256^3), then the two-warp shapes; for half storage row tiles first (whose 128-cell rows step 1.26x faster in row tiles),
-// then row segments in three consumer groups; then the register kernels; the register kernel for double storage (whose step is bound by the
-// double-precision pipe, which the register kernel's 4 warps per scheduler keep busier).
-static int default_variant(const rlb_ctx* c) {
-  static const int pref_f32[] = {19, 16, 15, 18, 17, 5, 12, 4, 13, 8, 6, 9, 7};
-  static const int pref_f16[] = {12, 16, 15, 13, 4, 8, 6, 5, 9, 7};
-  const int* pref = c->prm.storage == RLB_F32 ? pref_f32 : pref_f16;
-  const int n = c->prm.storage == RLB_F32 ? (int)(sizeof(pref_f32) / sizeof(int)) : (int)(sizeof(pref_f16) / sizeof(int));
-  if (c->prm.storage != RLB_F64)
-    for (int k = 0; k < n; ++k) {
-      // pipelined shapes only where the lattice's rows fill their tiles (rows_fit / rows_fit_solo
-      // for row tiles, pipe_fits for row segments); a forced variant may still run on any lattice
-      // it can take
-      if (pref[k] >= kNumRegVariants) {
-        PipeLayout lay;
-        if (!pipe_layout(pref[k], c->q, (int)c->elem, c->smem_per_sm, c->smem_optin, &lay)) continue;
-        const int elem = (int)c->elem;
-        const bool one = elem == 4 && !lay.split;  // one warp per float cell
-        bool fits = lay.rows ? (one ? rows_fit(c->sp.nx, lay.tx, elem, c->sp.bc[0], vmax_x(c))
-                                    : rows_fit_solo(c->sp.nx, lay.tx, elem, c->sp.bc[0], vmax_x(c)))
-                             : pipe_fits(c->sp.nx, lay.tx, elem, fill_eighths(lay, elem));
-        // 96-cell row tiles only where the rows fill them exactly (96-, 48- and 32-cell rows)
-        if (lay.tx == 96) fits = fits && (96 / c->sp.nx) * c->sp.nx == 96;
-        if (!fits) continue;
-      }
-      if (variant_available(c, pref[k])) return pref[k];
+// The row-tile variant whose tiles the lattice's rows fill best (at least 3/4 of the lanes), -1 if none.
+// Equal fills go to the first in an order measured on GB300: float 128-cell tiles (64^3 57 us a step
+// against 62 in 192-cell tiles, 128^3 351 against 440), then 192 (48^3 29 us against 32 in 96-cell
+// tiles, 96^3 170 against 171), half storage, whose copies are half as long, 192 and 256 (64^3 48 us
+// against 54 in 128-cell tiles, 128^3 315 against 335, 192^3 1.09 ms against 1.39 on the register kernel).
+// Tiles fewer than the SMs would leave some idle: then the narrowest.
+static int best_row_tiles(const rlb_ctx* c) {
+  static const int order_f32[] = {16, 22, 19, 21, 23}, order_f16[] = {22, 23, 21, 12, 19}, narrow[] = {19, 12, 16, 21, 22, 23};
+  const bool f32 = c->prm.storage == RLB_F32;
+  for (int pass = 0; pass < 2; ++pass) {
+    const int* order = pass ? narrow : (f32 ? order_f32 : order_f16);
+    int best = -1, cells = 0, width = 1;  // of the best so far: cells per tile, tile width
+    for (int k = 0; k < (pass ? 6 : 5); ++k) {
+      if (order[k] == (f32 ? 12 : 16)) continue;  // the slower of the two 128-cell shapes
+      PipeLayout lay;
+      if (!pipe_layout(order[k], c->q, (int)c->elem, c->smem_per_sm, c->smem_optin, &lay)) continue;
+      if (!rows_fit(c->sp.nx, lay.tx, (int)c->elem, c->sp.bc[0], vmax_x(c)) || !variant_available(c, order[k])) continue;
+      if (!pass && pipe_tile_count(c->sp.nx, c->sp.ny, c->sp.nz, lay.tx, 1) < c->sms) continue;
+      const int used = lay.tx / c->sp.nx * c->sp.nx;
+      if (best < 0 || used * width > cells * lay.tx) best = order[k], cells = used, width = lay.tx;
     }
+    if (best >= 0) return best;
+  }
+  return -1;
+}
+
+// The variant rlb_step uses unless asked otherwise.  Double storage, whose step is bound by the
+// double-precision pipe: the register kernels, which keep it busiest (small lattices: the team kernel).
+// Float and half storage: row tiles, then row segments (256^3 float: 2.85 ms a step against 3.70 on the register
+// kernels; narrower segments measured slower than those), then the register kernels (small lattices:
+// the team kernel).
+static int default_variant(const rlb_ctx* c) {
+  if (c->prm.storage != RLB_F64) {
+    const int rows = best_row_tiles(c);
+    if (rows >= 0) return rows;
+    const int seg = 15;
+    PipeLayout lay;
+    if (pipe_layout(seg, c->q, (int)c->elem, c->smem_per_sm, c->smem_optin, &lay) &&
+        pipe_fits(c->sp.nx, lay.tx, (int)c->elem, fill_eighths(lay, (int)c->elem)) && variant_available(c, seg))
+      return seg;
+  }
   return small_for_team(c) ? kTeamVariant : (c->prm.storage == RLB_F32 ? 3 : (c->prm.storage == RLB_F16DEV ? 2 : 0));
 }
 

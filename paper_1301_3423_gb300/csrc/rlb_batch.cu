@@ -140,7 +140,7 @@ static int member_mode(const rlb_batch* b, const StepParams& p, int v, const Pip
   if (!is_pipe(v)) return 0;
   const int vmax = b->order == 3 ? Quad3::VMAX_X : Quad2::VMAX_X;
   const int elem = elem_of(b->storage);
-  const bool seg = lay.tx != 96 && pipe_fits(p.nx, lay.tx, elem, fill_eighths(lay, elem));
+  const bool seg = (lay.tx == 64 || lay.tx == 128) && pipe_fits(p.nx, lay.tx, elem, fill_eighths(lay, elem));
   const bool rows = lay.rows && rows_fit(p.nx, lay.tx, elem, p.bc[0], vmax);
   if (lay96.tx == 96 && rows_fit(p.nx, 96, elem, p.bc[0], vmax) &&
       (!rows || row_tile_fill(p.nx, 96) * lay.tx > row_tile_fill(p.nx, lay.tx) * 96))
@@ -152,7 +152,7 @@ static int member_mode(const rlb_batch* b, const StepParams& p, int v, const Pip
 // The 96-cell row-tile variant with the warps of 128-cell row-tile variant v (-1 if none).
 static int rows96_sibling(int v) {
   if (!is_pipe(v)) return -1;
-  const PipeConfig& c = kPipeConfigs[v - kNumRegVariants];
+  const PipeConfig& c = pipe_config(v);
   if (!c.rows || c.tx != 128) return -1;
   for (int k = 0; k < kNumPipeConfigs; ++k) {
     const PipeConfig& d = kPipeConfigs[k];
@@ -167,7 +167,7 @@ static int rows96_sibling(int v) {
 // row-segment members in); v itself if it has no row tiles, -1 if none exists.
 static int segment_sibling(int v) {
   if (!is_pipe(v)) return v;
-  const PipeConfig& c = kPipeConfigs[v - kNumRegVariants];
+  const PipeConfig& c = pipe_config(v);
   if (!c.rows) return v;
   for (int k = 0; k < kNumPipeConfigs; ++k) {
     const PipeConfig& d = kPipeConfigs[k];

@@ -28,16 +28,27 @@ struct PipeConfig {
 // one consumer group, in the order of the stage's uses like every producer: a parity wait then
 // always refers to the phase it means.  With as many stages as groups each group refills its one
 // stage while the other groups compute.
+// A bulk copy takes some 45 clocks of an SM whatever its length (measured: 39 to 47 M copies/s and SM
+// from 132 to 528 bytes each), so the wide shapes copy the most per instruction that their stages
+// allow, and eight producer warps keep the copies going while four consumers' worth of registers would
+// only wait (256^3 float: 4 producers 3.03 ms, 8 2.91, 12 with 80 registers a thread 3.09).
 constexpr PipeConfig kPipeConfigs[] = {
     {128, 8, 1, 8, 0, 1}, {128, 8, 1, 4, 0, 1},  {64, 8, 1, 8, 0, 1},  {64, 4, 1, 4, 0, 1},
     {128, 8, 1, 6, 0, 1}, {64, 8, 1, 4, 0, 1},   {128, 4, 1, 4, 0, 1}, {64, 2, 1, 4, 0, 1},
-    {128, 8, 1, 4, 1, 1}, {128, 8, 1, 8, 1, 1},  {128, 4, 1, 4, 1, 1}, {128, 12, 1, 4, 0, 0},
-    {128, 12, 1, 4, 1, 0}, {128, 12, 1, 2, 0, 0}, {128, 12, 1, 2, 1, 0}, {96, 12, 1, 4, 1, 0}};
+    {128, 8, 1, 4, 1, 1}, {128, 8, 1, 8, 1, 1},  {128, 4, 1, 4, 1, 1}, {128, 12, 1, 8, 0, 0},
+    {128, 12, 1, 8, 1, 0}, {128, 12, 1, 2, 0, 0}, {128, 12, 1, 2, 1, 0}, {96, 12, 1, 8, 1, 0}};
+// Wider row tiles, numbered after the team kernel.
+constexpr PipeConfig kWideConfigs[] = {{160, 10, 1, 8, 1, 0}, {192, 12, 1, 8, 1, 0}, {256, 16, 1, 4, 1, 0}};
 constexpr int kNumPipeConfigs = sizeof(kPipeConfigs) / sizeof(kPipeConfigs[0]);
 // Variant after the pipelined shapes: the team kernel (rlb_team.cuh), for every storage and lattice.
 constexpr int kTeamVariant = kNumRegVariants + kNumPipeConfigs;
-constexpr int kNumVariantsTotal = kTeamVariant + 1;
-constexpr bool is_pipe(int v) { return v >= kNumRegVariants && v < kTeamVariant; }
+constexpr int kNumWideConfigs = sizeof(kWideConfigs) / sizeof(kWideConfigs[0]);
+constexpr int kNumVariantsTotal = kTeamVariant + 1 + kNumWideConfigs;
+constexpr bool is_pipe(int v) { return v >= kNumRegVariants && v != kTeamVariant && v < kNumVariantsTotal; }
+// The shape of pipelined variant v.
+constexpr const PipeConfig& pipe_config(int v) {
+  return v < kTeamVariant ? kPipeConfigs[v - kNumRegVariants] : kWideConfigs[v - kTeamVariant - 1];
+}
 constexpr int kTeamWarps = 4;   // warps that share a cell
 constexpr int kTeamCells = 32;  // cells per tile
 // Resident blocks per SM the team kernels' registers are cut to: 6 x 4 warps for float (80 registers),
@@ -45,10 +56,13 @@ constexpr int kTeamCells = 32;  // cells per tile
 template <class A>
 constexpr int kTeamBlocks = sizeof(A) == 8 ? 3 : 6;
 constexpr int kPipeMaxStages = 16;
-constexpr int kPipeMaxConsumerWarps = 12;
+constexpr int kPipeMaxConsumerWarps = 16;
 constexpr int kPipeMaxProducerWarps = 12;
-constexpr int kPipeMaxWarps = 16;  // consumers + producers: the launch bound of k_step_pipe (128 registers)
-constexpr int kPipeHeaderBytes = 1024;  // mbarriers (2 x 16 x 8 B) and the per-population velocity table
+// Consumers + producers, the launch bound of k_step_pipe: 20 warps of 96 registers for float and half
+// storage, 16 of 128 for double (whose cells need more).
+constexpr int pipe_max_warps(int elem) { return elem == 8 ? 16 : 20; }
+constexpr int kPipeChunks = 4;  // chunks of populations per stage, each with its own barriers
+constexpr int kPipeHeaderBytes = 1536;  // mbarriers (2 x 16 x 4 x 8 B) and the per-population velocity table
 constexpr int kPipeXchgBytesPerPair = 2 * 2 * 13 * 32 * 4;  // partial moments a consumer warp pair exchanges
 // Bytes of slack before and after every population buffer: the pipelined kernel's copies of a row
 // segment next to a lattice end may start up to one granule before the row and end up to one tile

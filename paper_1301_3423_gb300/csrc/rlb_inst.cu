@@ -78,6 +78,13 @@ cudaError_t pipe_step(const void* src, void* dst, const StepParams& p, const Pip
                       int rows, int split, int grid, int threads, int smem, cudaStream_t s) {
   if (rows) {
     if (tx == 96) return RLB_RFN(pipe, 96)(src, dst, p, pp, status, split, grid, threads, smem, s);
+#if RLB_WIDE
+    if (tx == 160) return RLB_RFN(pipe, 160)(src, dst, p, pp, status, split, grid, threads, smem, s);
+    if (tx == 192) return RLB_RFN(pipe, 192)(src, dst, p, pp, status, split, grid, threads, smem, s);
+#endif
+#if RLB_WIDE256
+    if (tx == 256) return RLB_RFN(pipe, 256)(src, dst, p, pp, status, split, grid, threads, smem, s);
+#endif
     if (tx != 128) return cudaErrorInvalidValue;
     return RLB_RFN(pipe, 128)(src, dst, p, pp, status, split, grid, threads, smem, s);
   }
@@ -89,6 +96,13 @@ cudaError_t pipe_batch_step(const BatchMember* m, const int* tm, int launch, con
                             int rows, int split, int walls, int grid, int threads, int smem, cudaStream_t s) {
   if (rows) {
     if (tx == 96) return RLB_RFN(pipe_batch, 96)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
+#if RLB_WIDE
+    if (tx == 160) return RLB_RFN(pipe_batch, 160)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
+    if (tx == 192) return RLB_RFN(pipe_batch, 192)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
+#endif
+#if RLB_WIDE256
+    if (tx == 256) return RLB_RFN(pipe_batch, 256)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
+#endif
     if (tx != 128) return cudaErrorInvalidValue;
     return RLB_RFN(pipe_batch, 128)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
   }

@@ -54,8 +54,9 @@ cudaError_t launch_pipe_batch(const BatchMember* m, const int* tm, int launch, c
   return cudaGetLastError();
 }
 
-// One warp per float cell exists for float storage with 128-cell tiles and 96-cell row tiles.
-constexpr bool kOneWarp = std::is_same<S, StoreF32>::value && (RLB_INST_TX == 128 || RLB_INST_TX == 96);
+// One warp per float cell exists for float storage from 96-cell tiles up.
+constexpr bool kOneWarp = std::is_same<S, StoreF32>::value && RLB_INST_TX >= 96;
+constexpr bool kWide = RLB_INST_TX > 128;  // one warp per float cell only
 }  // namespace
 
 // One time step of every active batch member on the pipelined kernel (walls: some member has
@@ -71,8 +72,11 @@ cudaError_t RLB_PIPE_FN(pipe_batch, RLB_INST_TX)(const BatchMember* m, const int
   } else if (!split && std::is_same<S, StoreF32>::value) {
     return cudaErrorInvalidValue;
   }
+  if constexpr (kOneWarp && kWide) return cudaErrorInvalidValue;
+  else {
   if (walls) return launch_pipe_batch<true, false>(m, tm, launch, pp, timeout, grid, threads, smem, s);
   return launch_pipe_batch<false, false>(m, tm, launch, pp, timeout, grid, threads, smem, s);
+  }
 }
 
 // One time step of the whole lattice in one launch, compiled with the bounce-back patch only for
@@ -87,7 +91,10 @@ cudaError_t RLB_PIPE_FN(pipe, RLB_INST_TX)(const void* src, void* dst, const Ste
   } else if (!split && std::is_same<S, StoreF32>::value) {
     return cudaErrorInvalidValue;
   }
+  if constexpr (kOneWarp && kWide) return cudaErrorInvalidValue;
+  else {
   if (p.has_wall) return launch_pipe<true, false>(src, dst, p, pp, status, grid, threads, smem, s);
   return launch_pipe<false, false>(src, dst, p, pp, status, grid, threads, smem, s);
+  }
 }
 }  // namespace rlb

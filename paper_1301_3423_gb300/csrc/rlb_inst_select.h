@@ -53,7 +53,10 @@ constexpr int kVariants = kFloat ? kNumVariants : 1;
 RLB_DECLARE_PIPE(64)
 RLB_DECLARE_PIPE(128)
 #undef RLB_DECLARE_PIPE
-// ... and with row tiles (RLB_INST_ROWS = 1), tile widths 128 and 96.
+// ... and with row tiles (RLB_INST_ROWS = 1), tile widths 128, 96 and the wide ones that are built
+// (pipe_built).
+#define RLB_WIDE (RLB_INST_STORAGE != 0)
+#define RLB_WIDE256 (RLB_INST_STORAGE == 2 || (RLB_INST_STORAGE == 1 && RLB_INST_ORDER == 2))
 #define RLB_RFN(fn, tx) RLB_CAT7(fn, _o, RLB_INST_ORDER, _s, RLB_INST_STORAGE, _r, tx)
 #define RLB_DECLARE_ROWS(tx)                                                                                   \
   cudaError_t RLB_RFN(pipe, tx)(const void* src, void* dst, const StepParams& p, const PipeParams& pp, int* status, \
@@ -63,6 +66,9 @@ RLB_DECLARE_PIPE(128)
                                       cudaStream_t s);
 RLB_DECLARE_ROWS(128)
 RLB_DECLARE_ROWS(96)
+RLB_DECLARE_ROWS(160)
+RLB_DECLARE_ROWS(192)
+RLB_DECLARE_ROWS(256)
 #undef RLB_DECLARE_ROWS
 
 // Team kernels (rlb_inst_team.cu).

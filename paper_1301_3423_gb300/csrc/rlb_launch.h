@@ -76,22 +76,11 @@ inline bool rows_possible(int nx, int tx, int elem, int bc_x, int vmax_x) {
   return bc_x == kPeriodic && nx <= tx && nx >= vmax_x && nx % (16 / elem) == 0;
 }
 
-// ... and suit it when the tile's G = tx / nx rows use at least 3/4 of its lanes (the batch's
-// rule: in the batched mix of 32- to 128-cell rows every such member stepped faster in row tiles
-// than on the register kernels).
+// ... and suit it when the tile's G = tx / nx rows use at least 3/4 of its lanes (in a batched mix of
+// 32- to 128-cell rows every such member stepped faster in row tiles than on the register kernels; a
+// 96-cell row per 128-cell tile ran 1.07x faster).
 inline bool rows_fit(int nx, int tx, int elem, int bc_x, int vmax_x) {
   return rows_possible(nx, tx, elem, bc_x, vmax_x) && 4 * (tx / nx) * nx >= 3 * tx;
-}
-
-// A single lattice's rule for layouts with two warps per float cell and half storage: several
-// rows per tile (G >= 2) at 3/4 of the lanes, or one row that fills the tile (measured on GB300
-// alone: 32-, 48- and 64-cell rows as fast as or faster than the register kernels, 128-cell rows
-// as fast as row segments with float storage and 1.26x faster with half storage, while one 96-cell
-// row per tile ran 1.4x slower than the register kernels).  One warp per float cell takes rows_fit
-// (a 96-cell row per tile ran 1.07x faster than the register kernels).
-inline bool rows_fit_solo(int nx, int tx, int elem, int bc_x, int vmax_x) {
-  if (!rows_fit(nx, tx, elem, bc_x, vmax_x)) return false;
-  return tx / nx >= 2 || nx == tx;
 }
 
 // Tiles of one lattice: row tiles (groups of tx / nx rows) or tx-cell row segments.
@@ -103,9 +92,16 @@ inline long long pipe_tile_count(int nx, int ny, int nz, int tx, int rows) {
   return (long long)((nx + tx - 1) / tx) * ny * nz;
 }
 
+// Tile widths above 128 are built for the float storages, 256 only where two stages of it fit (half
+// storage, and the second order's 66 float populations).
+constexpr bool pipe_built(int tx, int q, int elem) {
+  return tx <= 128 || (elem < 8 && (tx < 256 || q * elem < 128 * 4));
+}
+
 inline bool pipe_layout(int v, int q, int elem, int smem_per_sm, int smem_optin, PipeLayout* out) {
   if (!is_pipe(v)) return false;
-  const PipeConfig& cf = kPipeConfigs[v - kNumRegVariants];
+  const PipeConfig& cf = pipe_config(v);
+  if (!pipe_built(cf.tx, q, elem)) return false;
   const int A = 16 / elem;
   const long long stage = (long long)q * (cf.tx + A) * elem;
   long long budget = smem_per_sm / cf.ctas_per_sm - 1024;
@@ -115,7 +111,7 @@ inline bool pipe_layout(int v, int q, int elem, int smem_per_sm, int smem_optin,
   const int groups = cf.cons_warps / wpt;
   if (groups < 1 || cf.cons_warps % wpt != 0 || cf.producers < 1 || cf.producers > q) return false;
   if (cf.producers > kPipeMaxProducerWarps || cf.cons_warps > kPipeMaxConsumerWarps ||
-      cf.cons_warps + cf.producers > kPipeMaxWarps)
+      cf.cons_warps + cf.producers > pipe_max_warps(elem))
     return false;
   const long long xchg = split ? (long long)cf.cons_warps / 2 * kPipeXchgBytesPerPair : 0;
   long long fit = (budget - kPipeHeaderBytes - xchg) / stage;

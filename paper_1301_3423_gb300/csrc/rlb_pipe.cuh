@@ -32,8 +32,13 @@
 // tile.  NSTAGE is a multiple of the group count, so each stage is read by one group, and every
 // producer and that group take the stage's uses in order: when either waits for use u of a stage,
 // use u - 1 is complete and use u + 1 cannot be, and the parity of u names the right phase.
-// full[s] completes when every producer has arrived for the stage's tile and its copies have
-// landed; empty[s] when every consumer warp of that tile has finished reading it.  Every wait is
+// A stage is one chunk of populations, or four (row segments, one warp per float cell), with a barrier
+// pair each: full[s][c] completes when the chunk's producers have arrived for the stage's tile and
+// their copies have landed, empty[s][c] when every consumer warp of that tile has read the chunk for
+// the last time.  Moments and collision go through the chunks in order, so the next tile's first chunk
+// is on its way while the last is still being collided, and its moments start before its last chunk
+// has landed.  (256^3 float step, 8 producers: 2.82 ms in four chunks, 2.91 in one; row tiles, whose
+// tiles refill with one copy per population: 128^3 0.377 ms in four, 0.352 in one.)  Every wait is
 // bounded (kPipeWaitNs); a wait that runs out counts in status[kStatusTimeout], and the producer
 // then waits (bounded) for the copies it has in flight before it returns.
 #pragma once
@@ -44,7 +49,8 @@
 
 namespace rlb {
 
-constexpr int kPipeMaxThreads = kPipeMaxWarps * 32;
+template <class S>
+constexpr int kPipeMaxThreads = sizeof(typename S::T) == 8 ? 16 * 32 : 20 * 32;  // pipe_max_warps
 constexpr unsigned long long kPipeWaitNs = 2000000000ull;  // 2 s
 
 // Geometry of one staged row for storage S and tile width TX.
@@ -135,6 +141,18 @@ struct DpSplit {
   static constexpr int value = find();
 };
 
+// A stage's populations in chunks, each with its own pair of barriers: each filled
+// by its own producers as soon as it is read.  Whole mirror pairs.
+template <class L, int NCH>
+struct ChunkSize {
+  static constexpr int value = (L::Q / 2 + NCH - 1) / NCH * 2;
+};
+// Producers of chunk c of NCH among P.
+template <int NCH>
+__device__ __forceinline__ int chunk_producers(int c, int P) {
+  return P < NCH ? 1 : (P - c + NCH - 1) / NCH;
+}
+
 // Floats a consumer warp pair exchanges per tile: two buffers (alternate tiles) x two halves x 13
 // partial moments x 32 lanes.
 constexpr int kPipeXchgFloatsPerPair = kPipeXchgBytesPerPair / 4;
@@ -208,20 +226,25 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
   constexpr int kStageElems = L::Q * BX;
   constexpr bool DEV = std::is_same<S, StoreF16Dev>::value;
   static_assert(TX % 32 == 0 && TX >= 32, "tile width");
+  // Row segments with one warp per float cell release their stage chunk by chunk while they collide;
+  // the others have one chunk, the stage.
+  constexpr bool EARLY = PACKED && !SPLIT && !ROWS;
+  constexpr int NCH = EARLY ? kPipeChunks : 1, CH = ChunkSize<L, NCH>::value;
 
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t* full = reinterpret_cast<uint64_t*>(smem);
-  uint64_t* empty = full + kPipeMaxStages;
-  char4* sv = reinterpret_cast<char4*>(smem + 2 * 8 * kPipeMaxStages);
+  uint64_t* empty = full + kPipeMaxStages * kPipeChunks;
+  char4* sv = reinterpret_cast<char4*>(smem + 2 * 8 * kPipeMaxStages * kPipeChunks);
   T* const stage0 = reinterpret_cast<T*>(smem + kPipeHeaderBytes);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cons_warps = pp.groups * WPT;  // warps [0, cons_warps) consume, the next pp.producers produce
   if (threadIdx.x == 0) {
-    for (int s = 0; s < pp.nstage; ++s) {
-      mbar_init(&full[s], pp.producers);
-      mbar_init(&empty[s], WPT);
-    }
+    for (int s = 0; s < pp.nstage; ++s)
+      for (int c = 0; c < NCH; ++c) {
+        mbar_init(&full[s * NCH + c], chunk_producers<NCH>(c, pp.producers));
+        mbar_init(&empty[s * NCH + c], WPT);
+      }
     static_for<L::Q>([&](auto I) {
       constexpr int i = decltype(I)::value;
       constexpr signed char vx = L::VX[i], vy = L::VY[i], vz = L::VZ[i];
@@ -233,23 +256,19 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
   const long long G = gridDim.x;
 
   if (warp >= cons_warps) {
-    // ---- producer warps, a team over every tile: producer w copies populations i = w, w + P, ...
-    // (lane l takes i = l P + w, then i + 32 P), one bulk copy each (a few at a periodic x end),
-    // and arrives once per tile on the stage's full barrier with its share of the bytes
+    // ---- producer warps, a team over every tile: producer w copies chunk w mod 4 of the populations
+    // (with more than four producers they share a chunk, with fewer one takes several), lane l one
+    // population, with one bulk copy each (a few at a periodic x end), and arrives once per tile and
+    // chunk on its full barrier with its share of the bytes
     const int pw = warp - cons_warps;
     const int P = pp.producers;
-    const int mine = (L::Q - pw + P - 1) / P;  // populations of this producer
     if (tiles.debug() & kDebugStallProducers) return;  // testing: nothing arrives, every wait runs out
     int k = 0;
     bool ok = true;
-    for (;; ++k) {
+    for (; ok; ++k) {
       const long long t = blockIdx.x + (long long)k * G;
       if (t >= pp.ntiles) break;
       const int s = k % pp.nstage;
-      if (k >= pp.nstage && !mbar_wait(&empty[s], (uint32_t)((k / pp.nstage) - 1) & 1u)) {
-        ok = false;
-        break;
-      }
       const auto tr = tiles.at(t, tiles.member(t));
       const StepParams& p = tr.p;
       // row tiles: rows r0 .. r0 + gt - 1 of the lattice, gt * nx elements per population
@@ -258,9 +277,6 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
       const int r0 = ROWS ? tr.lt * rpt : 0;
       const int gt = ROWS ? min(rpt, nrows - r0) : 1;
       const uint32_t pop_bytes = ROWS ? (uint32_t)(gt * p.nx * (int)sizeof(T)) : (uint32_t)Sh::ROW_BYTES;
-      if (lane == 0) mbar_arrive_expect_tx(&full[s], tr.active ? (uint32_t)mine * pop_bytes : 0u);
-      __syncwarp();
-      if (!tr.active) continue;
       const T* __restrict__ src = tr.src;
       const int segs = ROWS ? 1 : (p.nx + TX - 1) / TX;
       const int seg = ROWS ? 0 : tr.lt % segs, row = ROWS ? r0 : tr.lt / segs;
@@ -272,19 +288,32 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
       // read from the buffer's start instead (the byte count of the stage stays the same)
       const long long lo = -(long long)(kPopGuardBytes / sizeof(T));
       const long long hi = (long long)L::Q * p.cells + kPopGuardBytes / sizeof(T);
-      auto copy = [&](T* d, long long from, int n) {
+      auto copy = [&](T* d, long long from, int n, uint64_t* bar) {
         if (from < lo || from + n > hi) {
           atomicAdd(&tr.status[kStatusBounds], 1);
           from = 0;
         }
-        bulk_g2s(d, src + from, (uint32_t)(n * sizeof(T)), &full[s]);
+        bulk_g2s(d, src + from, (uint32_t)(n * sizeof(T)), bar);
       };
-      if constexpr (ROWS) {
-        // each run of consecutive source rows of population i with one copy of whole rows
-        for (int i = lane * P + pw; i < L::Q; i += 32 * P) {
-          const char4 v = sv[i];
-          const long long base = (long long)i * p.cells;
-          T* d = st + i * BX;
+      for (int c = pw % NCH; c < NCH; c += P < NCH ? P : NCH) {
+        uint64_t* const bar = &full[s * NCH + c];
+        const int share = chunk_producers<NCH>(c, P);  // producers of this chunk; this one's number is first
+        const int first = P < NCH ? 0 : pw / NCH;
+        const int end = min((c + 1) * CH, L::Q);
+        const int mine = max(0, (end - c * CH - first + share - 1) / share);
+        if (k >= pp.nstage && !mbar_wait(&empty[s * NCH + c], (uint32_t)((k / pp.nstage) - 1) & 1u)) ok = false;
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        if (lane == 0) mbar_arrive_expect_tx(bar, tr.active ? (uint32_t)mine * pop_bytes : 0u);
+        __syncwarp();
+        if (!tr.active) continue;
+        for (int j = lane; j < mine; j += 32) {
+        const int i = c * CH + first + j * share;
+        const char4 v = sv[i];
+        const long long plane = (long long)i * p.cells;
+        T* const d = st + i * BX;
+        if constexpr (ROWS) {
+          // each run of consecutive source rows with one copy of whole rows
           int r = 0, yr = y, zr = z;
           long long run0 = 0, next = -1;
           int runlen = 0;
@@ -292,7 +321,7 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
             const long long sr = (long long)pipe_src_row(zr - v.z, p.nz, p.bc[2]) * p.ny +
                                  pipe_src_row(yr - v.y, p.ny, p.bc[1]);
             if (sr != next) {
-              if (runlen > 0) copy(d + (r - runlen) * p.nx, base + run0 * p.nx, runlen * p.nx);
+              if (runlen > 0) copy(d + (r - runlen) * p.nx, plane + run0 * p.nx, runlen * p.nx, bar);
               run0 = sr;
               runlen = 0;
             }
@@ -303,17 +332,11 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
               ++zr;
             }
           }
-          copy(d + (r - runlen) * p.nx, base + run0 * p.nx, runlen * p.nx);
-        }
-        continue;
-      }
-      for (int i = lane * P + pw; i < L::Q; i += 32 * P) {
-        const char4 v = sv[i];
-        const int ys = pipe_src_row(y - v.y, p.ny, p.bc[1]);
-        const int zs = pipe_src_row(z - v.z, p.nz, p.bc[2]);
-        const long long row0 = (long long)i * p.cells + ((long long)zs * p.ny + ys) * p.nx;
+          copy(d + (r - runlen) * p.nx, plane + run0 * p.nx, runlen * p.nx, bar);
+        } else {
+        const long long row0 =
+            plane + ((long long)pipe_src_row(z - v.z, p.nz, p.bc[2]) * p.ny + pipe_src_row(y - v.y, p.ny, p.bc[1])) * p.nx;
         const int xs = (x0 - v.x) & ~(AL - 1);  // round down to a granule (two's complement: floor)
-        T* d = st + i * BX;
         if (xperiodic && (xs < 0 || xs + BX > p.nx)) {
           // split [xs, xs + BX) at multiples of nx; each piece is whole granules of one period
           int a = xs;
@@ -321,13 +344,15 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
           while (a < e) {
             const int per = (a >= 0) ? a / p.nx : -((-a + p.nx - 1) / p.nx);
             const int pe = min(e, (per + 1) * p.nx);
-            copy(d + (a - xs), row0 + (a - per * p.nx), pe - a);
+            copy(d + (a - xs), row0 + (a - per * p.nx), pe - a, bar);
             a = pe;
           }
         } else {
           // x beyond the ends reads neighbouring memory (guard bytes around every buffer); the
           // consumer patches those cells
-          copy(d, row0 + xs, BX);
+          copy(d, row0 + xs, BX, bar);
+        }
+        }
         }
       }
     }
@@ -335,7 +360,12 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
       if (lane == 0) atomicAdd(tiles.timeout_word(), 1);
       // let the copies already issued land before the block's shared memory goes away (each stage's
       // latest use among the last nstage tiles)
-      for (int j = max(0, k - pp.nstage); j < k; ++j) mbar_wait(&full[j % pp.nstage], (uint32_t)(j / pp.nstage) & 1u);
+      for (int j = max(0, k - 1 - pp.nstage); j < k - 1; ++j)
+        for (int c = pw % NCH; c < NCH; c += P < NCH ? P : NCH)
+          mbar_wait(&full[j % pp.nstage * NCH + c], (uint32_t)(j / pp.nstage) & 1u);
+      // (with fewer than four producers also the chunks of the tile it gave up in)
+      for (int c = pw % NCH; P < NCH && c < NCH; c += P)
+        mbar_wait(&full[(k - 1) % pp.nstage * NCH + c], (uint32_t)((k - 1) / pp.nstage) & 1u);
     }
     return;
   }
@@ -363,14 +393,33 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
       const long long tn = t + (long long)pp.groups * G;
       if (tn < pp.ntiles) next_member = tiles.member(tn);
     }
+    const uint32_t parity = (uint32_t)(k / pp.nstage) & 1u;
+    bool late = false;  // a wait ran out
+    auto wait_chunk = [&](int c) { late = !mbar_wait(&full[s * NCH + c], parity) || late; };
+    auto release = [&](int c) {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[s * NCH + c]);
+    };
+    auto wait_all = [&] {
+#pragma unroll
+      for (int c = 0; c < NCH; ++c) wait_chunk(c);
+    };
+    auto release_all = [&] {
+      __syncwarp();
+      if (lane < NCH) mbar_arrive(&empty[s * NCH + lane]);
+    };
+    // true (in every lane) once a wait has run out: the warp counts it and leaves
+    auto gave_up = [&]() -> bool {
+      if (!__any_sync(0xffffffffu, late)) return false;
+      if (lane == 0) atomicAdd(tiles.timeout_word(), 1);
+      return true;
+    };
     // a batch works out the tile's cells and stage offsets (from the member's parameters in
     // memory) before the wait for the stage, so that their loads overlap it; a single lattice, whose
     // parameters are kernel arguments, waits first (measured 2% faster)
     if constexpr (!Tiles::kEarlyGeometry) {
-      if (!mbar_wait(&full[s], (uint32_t)(k / pp.nstage) & 1u)) {
-        if (lane == 0) atomicAdd(tiles.timeout_word(), 1);
-        return;
-      }
+      wait_chunk(0);
+      if (gave_up()) return;
     }
     const StepParams& p = tr.p;
     const T* __restrict__ src = tr.src;
@@ -423,17 +472,16 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
       else return i * BX + ((-L::VX[i]) % AL + AL) % AL;
     };
     if constexpr (Tiles::kEarlyGeometry) {
-      if (!mbar_wait(&full[s], (uint32_t)(k / pp.nstage) & 1u)) {
-        if (lane == 0) atomicAdd(tiles.timeout_word(), 1);
-        return;
-      }
+      wait_chunk(0);
+      if (gave_up()) return;
     }
     // a lattice that does not step, or a warp none of whose lanes holds a cell of the tile (the
     // last part of a tile of 96-cell rows, a ragged row end): release the stage and leave the issue
     // slots to the other warps (both warps of a float pair skip together)
     if (!tr.active || !__any_sync(0xffffffffu, valid)) {
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&empty[s]);
+      wait_all();
+      if (gave_up()) return;
+      release_all();
       continue;
     }
 
@@ -449,6 +497,10 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
       const bool near = (p.bc[1] == kBounceBack && (cl.y < L::VMAX_Y || cl.y >= p.ny - L::VMAX_Y)) ||
                         (p.bc[2] == kBounceBack && (cl.z < L::VMAX_Z || cl.z >= p.nz - L::VMAX_Z));
       patch = patch || (ROWS ? __any_sync(0xffffffffu, near) : near);
+    }
+    if (patch || !EARLY) {
+      wait_all();
+      if (gave_up()) return;
     }
     if (patch) {
       static_for<L::Q>([&](auto I) {
@@ -485,14 +537,56 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
         else S::template store<L, i>(out + (long long)i * p.cells, v, p);
       }
     };
-    if constexpr (!SPLIT) {
+    auto get2 = [&](auto I) -> float2 {
+      constexpr int i = decltype(I)::value;
+      return make_float2(get(ic<i>{}), get(ic<i + 1>{}));
+    };
+    const float c_dev = DEV ? p.half_nref : 0.f;
+    if constexpr (EARLY) {
+      // moments, waiting for each chunk of the stage as its first population is read
+      Mom<float> m = moments_f2<L, DEV>(
+          [&](auto I) -> float2 {
+            constexpr int i = decltype(I)::value;
+            if constexpr (i % CH == 0 && i > 0) wait_chunk(i / CH);
+            return get2(I);
+          },
+          c_dev);
+      if (gave_up()) return;
+      reload_barrier();
+      const Landau<float> lw = landau_step<float>(m, p);
+      const float Tl = lw.eps / (3.f * lw.n);
+      const float inv_tau = 1.f / tau_prime<float>(Tl, p);
+      const CollideCoef<L> q = collide_coef<L, DEV>(lw, Tl, inv_tau, c_dev);
+      // collision; each chunk goes back to the producers once it is read, if every lane has a frame
+      const bool all_ok = __all_sync(0xffffffffu, lw.ok);
+      const bool put = valid && lw.ok;
+      collide_f2<L, DEV>(q, get2, [&](auto I, float2 v) {
+        constexpr int i = decltype(I)::value;
+        if (put) {
+          if constexpr (DEV) {
+            S::template store_dev<L, i>(out + (long long)i * p.cells, v.x, p);
+            S::template store_dev<L, i + 1>(out + (long long)(i + 1) * p.cells, v.y, p);
+          } else {
+            S::template store<L, i>(out + (long long)i * p.cells, v.x, p);
+            S::template store<L, i + 1>(out + (long long)(i + 1) * p.cells, v.y, p);
+          }
+        }
+        if constexpr ((i + 2) % CH == 0 || i + 2 == L::Q) {
+          if (all_ok) release(i / CH);
+        }
+      });
+      if (!all_ok) {
+        if (!lw.ok && valid) {
+          // no Landau frame: record it and stream the populations without collision
+          atomicAdd(&status[kStatusNonconv], 1);
+          static_for<L::Q>([&](auto I) { store(I, get(I)); });
+        }
+        release_all();
+      }
+      continue;
+    } else if constexpr (!SPLIT) {
       relax_cell<L, S, PACKED, true>(get, store, p, status, valid);
     } else {
-      auto get2 = [&](auto I) -> float2 {
-        constexpr int i = decltype(I)::value;
-        return make_float2(get(ic<i>{}), get(ic<i + 1>{}));
-      };
-      const float c_dev = DEV ? p.half_nref : 0.f;
       Mom<float> m = half == 0 ? moments_f2_part<L, DEV, 0, KS>(get2) : moments_f2_part<L, DEV, KS, L::NDP>(get2);
       // exchange the 13 partial sums with the partner warp (buffer iter & 1) and add them
       float* mine = xb + ((iter & 1) * 2 + half) * 13 * 32;
@@ -530,8 +624,7 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
         else collide_f2<L, DEV, KS, L::NDP>(q, get2, put2);
       }
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&empty[s]);
+    release_all();
   }
 }
 
@@ -586,7 +679,7 @@ struct BatchTiles {
 
 // One time step of one lattice.
 template <class L, class S, int TX, bool WALLS, bool ROWS, bool ONEWARP>
-__global__ void __launch_bounds__(kPipeMaxThreads, 1)
+__global__ void __launch_bounds__(kPipeMaxThreads<S>, 1)
     k_step_pipe(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
                 const __grid_constant__ StepParams p, const __grid_constant__ PipeParams pp,
                 int* __restrict__ status) {
@@ -598,7 +691,7 @@ __global__ void __launch_bounds__(kPipeMaxThreads, 1)
 // members' tiles.  A member's result is bitwise that of k_step_pipe on it alone.  Waits that run
 // out are counted in *timeout (the first member's status words).
 template <class L, class S, int TX, bool WALLS, bool ROWS, bool ONEWARP>
-__global__ void __launch_bounds__(kPipeMaxThreads, 1)
+__global__ void __launch_bounds__(kPipeMaxThreads<S>, 1)
     k_step_pipe_batch(const BatchMember* __restrict__ members, const int* __restrict__ tile_member, int launch,
                       const __grid_constant__ PipeParams pp, int* __restrict__ timeout) {
   using T = typename S::T;
