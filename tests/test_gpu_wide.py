@@ -41,9 +41,10 @@ def test_wide_row_tiles_equal_row_segments(order, storage, case):
 
 
 @pytest.mark.parametrize("bc", [(0, 0, 0), (1, 0, 0), (2, 2, 1)])
-def test_chunked_segments_with_cells_without_a_frame(bc):
-    """Cells without a Landau frame keep their stage whole (no early release): counted and streamed as
-    by the kernel that refills whole stages, over several tiles per block."""
+def test_chunked_segments_with_some_cells_without_a_frame(bc):
+    """Warps some of whose cells have no Landau frame keep their stage whole (no early release).  NaN in
+    a few cells leaves every cell that pulls from them without a frame: the same cells are counted and
+    streamed as by the kernel that refills whole stages, the others agree to the order of the sums."""
     from paper_1301_3423_gb300 import RLBError
     shape = (40, 24, 256)
     n, T, u = gen.smooth_random_fields(shape, seed=121, vmax=0.3, sigma_lnT=0.1, kmax=1)
@@ -53,8 +54,7 @@ def test_chunked_segments_with_cells_without_a_frame(bc):
             g.init(n, T, u)
             f = torch.empty((g.q,) + shape, dtype=torch.float64, device="cuda")
             g.populations(out=f)
-            f[:, 5:9, 3, 60:90] = 0
-            f[0, 5:9, 3, 60:90] = 1
+            f[:, 5:9, 3, 60:90] = float("nan")
             g.set_populations(f)
             g.step(1)
             with pytest.raises(RLBError) as e:
@@ -62,8 +62,30 @@ def test_chunked_segments_with_cells_without_a_frame(bc):
             counts.append(str(e.value))
             got.append(g.populations())
     assert counts[0] == counts[1]
-    scale = np.abs(got[1]).max(axis=(1, 2, 3), keepdims=True)
-    assert np.max(np.abs(got[0] - got[1]) / scale) < 4e-6  # one and two warps per cell sum in another order
+    a, b = got
+    assert np.array_equal(np.isnan(a), np.isnan(b))
+    scale = np.nanmax(np.abs(b), axis=(1, 2, 3), keepdims=True)
+    assert np.nanmax(np.abs(a - b) / scale) < 4e-6  # one and two warps per cell sum in another order
+
+
+def test_chunked_segments_without_any_frame():
+    """One population everywhere: every cell streams it unchanged, over several tiles per block.  Powers of
+    two, so that a lone population's null current rounds alike in every cell."""
+    from paper_1301_3423_gb300 import RLBError
+    shape = (40, 24, 256)
+    with RLB(shape, storage="f32", step_variant=15) as g:
+        x = (2.0 ** np.random.default_rng(5).integers(-3, 4, shape)).astype(np.float32)
+        f = torch.zeros((g.q,) + shape, dtype=torch.float64, device="cuda")
+        f[0] = torch.from_numpy(x).cuda()
+        g.set_populations(f)
+        g.step(1)
+        with pytest.raises(RLBError) as e:
+            g.sync()
+        assert "%d cell" % x.size in str(e.value)
+        p = g.populations()
+    from paper_1301_3423_gb300 import quadrature
+    v = quadrature(3)["v"][0]
+    assert np.array_equal(p[0], np.roll(x, (v[2], v[1], v[0]), axis=(0, 1, 2))) and not p[1:].any()
 
 
 @pytest.mark.parametrize("variant", [21, 22, 23])
