@@ -173,16 +173,32 @@ __constant__ VelTab<L> kVelTab = make_vel_tab<L>();
 
 // Pull offsets of one shell row (fixed y, z): for every population the constant offset plus the
 // row's y and z wrap (or clamp) shifts, worked out once per row by the warp's 32 lanes (four
-// populations each) into roff[Q]; the warp's cells then add only their x shift.  Lattices with
-// bounce-back walls take shell_row_offset per population instead.
-template <class L>
-__device__ __forceinline__ void shell_row_table(long long* roff, const Cell& cl, const StepParams& p) {
-  for (int i = threadIdx.x & 31; i < L::Q; i += 32) {
-    const int vy = kVelTab<L>.v[i][1], vz = kVelTab<L>.v[i][2];
-    long long o = p.off[i];
-    o += (long long)(src_coord_rt(cl.y, vy, p.ny, p.bc[1]) - (cl.y - vy)) * p.nx;
-    o += (long long)(src_coord_rt(cl.z, vz, p.nz, p.bc[2]) - (cl.z - vz)) * p.nxy;
-    roff[i] = o;
+// populations each) into roff[Q]; the warp's cells then add only their x shift.  A population that
+// comes from beyond a wall in y or z does so in the whole row: its offset is that of the cell's own
+// reversed population (I ^ 1: mirror pairs are adjacent), to which no x shift is added; bit i % 32 of
+// walled[i / 32] marks it.  (151 x 93 x 70 float lattice with walls on y, 28 % shell rows: with the wall
+// test per cell and population instead the shell kernel took 178 us beside the interior's 204.)
+template <class L, bool WALLS>
+__device__ __forceinline__ void shell_row_table(long long* roff, uint32_t (&walled)[4], const Cell& cl,
+                                                const StepParams& p) {
+  static_assert(L::Q <= 128, "four words of flags");
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int i = (threadIdx.x & 31) + 32 * k;
+    bool beyond = false;
+    if (i < L::Q) {
+      const int vy = kVelTab<L>.v[i][1], vz = kVelTab<L>.v[i][2];
+      long long o = p.off[i];
+      o += (long long)(src_coord_rt(cl.y, vy, p.ny, p.bc[1]) - (cl.y - vy)) * p.nx;
+      o += (long long)(src_coord_rt(cl.z, vz, p.nz, p.bc[2]) - (cl.z - vz)) * p.nxy;
+      if constexpr (WALLS) {
+        beyond = (p.bc[1] == kBounceBack && (unsigned)(cl.y - vy) >= (unsigned)p.ny) ||
+                 (p.bc[2] == kBounceBack && (unsigned)(cl.z - vz) >= (unsigned)p.nz);
+        if (beyond) o = (long long)(i ^ 1) * p.cells;
+      }
+      roff[i] = o;
+    }
+    walled[k] = WALLS ? __ballot_sync(0xffffffffu, beyond) : 0u;
   }
   __syncwarp();
 }
@@ -238,15 +254,33 @@ struct PullTab {
 #pragma unroll
     for (int j = 0; j <= 2 * L::VMAX_Z; ++j) z[j] = wrap(cl.z - (j - L::VMAX_Z), p.nz, p.bc[2]) * p.nxy;
   }
-  // index into the population buffer: plane offset of I (its mirror partner's beyond a wall) plus
-  // the in-plane index
+  // The velocity components that point beyond a wall of each axis, as bits (none on lattices without).
+  unsigned wx = 0, wy = 0, wz = 0;
+  __device__ __forceinline__ void find_walls(const Cell& cl, const StepParams& p) {
+    auto bits = [](int s, int n, int vmax) {  // components v with s - v outside 0 .. n - 1: bit v + vmax
+      const int lo = max(s + 1, -vmax), hi = min(s - n, vmax);
+      unsigned m = 0;
+      if (lo <= vmax) m |= ~0u << (lo + vmax) & ((2u << (2 * vmax)) - 1u);
+      if (hi >= -vmax) m |= (2u << (hi + vmax)) - 1u;
+      return m;
+    };
+    if (p.bc[0] == kBounceBack) wx = bits(cl.x, p.nx, L::VMAX_X);
+    if (p.bc[1] == kBounceBack) wy = bits(cl.y, p.ny, L::VMAX_Y);
+    if (p.bc[2] == kBounceBack) wz = bits(cl.z, p.nz, L::VMAX_Z);
+  }
+  // index into the population buffer: plane offset of I plus the in-plane index; with WALLS the cell's
+  // own value of the mirror partner where I points beyond a wall
   template <int I, bool WALLS>
   __device__ __forceinline__ long long index(const Cell& cl, const StepParams& p) const {
+    constexpr int vx = L::VX[I], vy = L::VY[I], vz = L::VZ[I];
     if constexpr (WALLS) {
-      if (beyond_wall<L, I>(cl, p)) return (long long)(I ^ 1) * p.cells + cl.c;
+      unsigned b = 0;
+      if constexpr (vx != 0) b |= wx & (1u << (vx + L::VMAX_X));
+      if constexpr (vy != 0) b |= wy & (1u << (vy + L::VMAX_Y));
+      if constexpr (vz != 0) b |= wz & (1u << (vz + L::VMAX_Z));
+      if (b) return (long long)(I ^ 1) * p.cells + cl.c;
     }
-    return (long long)I * p.cells +
-           (unsigned)(x[L::VX[I] + L::VMAX_X] + y[L::VY[I] + L::VMAX_Y] + z[L::VZ[I] + L::VMAX_Z]);
+    return (long long)I * p.cells + (unsigned)(x[vx + L::VMAX_X] + y[vy + L::VMAX_Y] + z[vz + L::VMAX_Z]);
   }
 };
 
@@ -724,24 +758,6 @@ __device__ __forceinline__ EqCoef<ORDER, A> eq_coef(A n, A T, A U0) {
   return c;
 }
 
-// Pull offset of population I from the cell's own index in a shell row: the constant offset plus
-// the y and z wrap (or clamp) shifts of the row, plus the x shift unless the warp's x segment is
-// interior; the cell's own reversed population beyond a bounce-back wall.
-template <class L, int I, bool WALLS>
-__device__ __forceinline__ long long shell_row_offset(const Cell& cl, const StepParams& p, const bool xfast) {
-  constexpr int vx = L::VX[I], vy = L::VY[I], vz = L::VZ[I];
-  if constexpr (WALLS) {
-    if (p.has_wall && beyond_wall<L, I>(cl, p)) return (long long)(I ^ 1) * p.cells;
-  }
-  long long o = p.off[I];
-  if constexpr (vy != 0) o += (long long)(src_coord<vy, false>(cl.y, p.ny, p.bc[1]) - (cl.y - vy)) * p.nx;
-  if constexpr (vz != 0) o += (long long)(src_coord<vz, false>(cl.z, p.nz, p.bc[2]) - (cl.z - vz)) * p.nxy;
-  if constexpr (vx != 0) {
-    if (!xfast) o += src_coord<vx, false>(cl.x, p.nx, p.bc[0]) - (cl.x - vx);
-  }
-  return o;
-}
-
 // The equilibrium as a polynomial in t per energy level l (p0 = p0_l):
 //   E(p0_l, t) = a_l + t (b_l + t (c_l + t d_l)),
 //   order 3: a = c00 + p0 c10 + p0^2 c20 + pref p0^3 x^3,  b = p0 c01 + p0^2 c11 + 3 pref p0^3 x^2 T,
@@ -1063,7 +1079,7 @@ struct StepShape {
 // kernel's warps lie in boundary rows, whose y and z shifts are the same for the whole warp; the
 // per-cell shell kernel (lattices shorter than the stencil reach) wraps every coordinate of every
 // cell.
-enum PullPath : int { kPathRow = 1, kPathEdge = 2, kPathShellRow = 3, kPathShellTab = 4 };
+enum PullPath : int { kPathRow = 1, kPathEdge = 2, kPathShellTab = 3 };
 
 // One cell's time step (pull, moments, Landau matching, equilibrium, collision, store).  Invalid
 // lanes (valid = false) carry a clamped in-range cell, compute and store nothing.
@@ -1071,16 +1087,15 @@ template <class L, class S, bool GENERAL, int VARIANT, int PATH, bool WALLS>
 __device__ __forceinline__ void step_cell(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
                                           const StepParams& p, int* __restrict__ status, const Cell cl,
                                           const bool valid, const bool row_fast = false,
-                                          const long long* __restrict__ roff = nullptr) {
+                                          const long long* __restrict__ roff = nullptr,
+                                          const uint32_t* walled = nullptr) {
   using A = typename S::A;
   using ST = typename S::T;
   constexpr bool PACKED = (VARIANT & 1) && std::is_same<A, float>::value;
   constexpr bool KEEP = StepShape<S, VARIANT>::kKeep;
   // Warp-uniform choice: a row warp whose segment is interior pulls with constant offsets; other
   // row warps wrap x only; shell cells resolve wrap / copy-out / bounce-back per population.
-  static_assert(PATH == kPathRow || PATH == kPathEdge || PATH == kPathShellRow || PATH == kPathShellTab,
-                "pull path");
-  static_assert(PATH != kPathShellTab || !WALLS, "the shell-row table has no bounce-back walls");
+  static_assert(PATH == kPathRow || PATH == kPathEdge || PATH == kPathShellTab, "pull path");
   const bool fast = PATH == kPathRow && row_fast;
   const ST* __restrict__ base = src + cl.c;
   ST* __restrict__ out = dst + cl.c;
@@ -1097,12 +1112,16 @@ __device__ __forceinline__ void step_cell(const typename S::T* __restrict__ src,
     constexpr int i = decltype(I)::value;
     if (fast) return ld(I, base + p.off[i]);
     if constexpr (PATH == kPathRow) return ld(I, base + x_row_offset<L, i, WALLS>(cl, p));
-    else if constexpr (PATH == kPathShellRow) return ld(I, base + shell_row_offset<L, i, WALLS>(cl, p, row_fast));
     else if constexpr (PATH == kPathShellTab) {
       constexpr int vx = L::VX[i];
       long long o = roff[i];
       if constexpr (vx != 0) {
-        if (!row_fast) o += src_coord<vx, false>(cl.x, p.nx, p.bc[0]) - (cl.x - vx);
+        bool shift = !row_fast;
+        if constexpr (WALLS) shift = shift && !(walled[i / 32] >> (i % 32) & 1u);
+        if (shift) {
+          if (WALLS && p.bc[0] == kBounceBack && (unsigned)(cl.x - vx) >= (unsigned)p.nx) o = (long long)(i ^ 1) * p.cells;
+          else o += src_coord<vx, false>(cl.x, p.nx, p.bc[0]) - (cl.x - vx);
+        }
       }
       return ld(I, base + o);
     }
@@ -1194,13 +1213,10 @@ __global__ void __launch_bounds__(32, 4 * StepShape<S, VARIANT>::kMinBlocks)
   cl.x = valid ? x : p.nx - 1;
   cl.c = (cl.z * p.ny + cl.y) * p.nx + cl.x;
   const bool xfast = x0 >= p.ix0 && min(x0 + 31, p.nx - 1) < p.ix0 + p.ixn;
-  if constexpr (WALLS) {
-    step_cell<L, S, false, VARIANT, kPathShellRow, WALLS>(src, dst, p, status, cl, valid, xfast);
-  } else {
-    __shared__ long long roff[L::Q];
-    shell_row_table<L>(roff, cl, p);
-    step_cell<L, S, false, VARIANT, kPathShellTab, false>(src, dst, p, status, cl, valid, xfast, roff);
-  }
+  __shared__ long long roff[L::Q];
+  uint32_t walled[4];
+  shell_row_table<L, WALLS>(roff, walled, cl, p);
+  step_cell<L, S, false, VARIANT, kPathShellTab, WALLS>(src, dst, p, status, cl, valid, xfast, roff, walled);
 }
 
 // Shell cells (rows whose y or z lies outside the interior box): z-boundary planes, then the
@@ -1306,13 +1322,10 @@ __global__ void __launch_bounds__(kStepThreads, StepShape<S, VARIANT>::kMinBlock
           cl.x = valid ? x : sp.nx - 1;
           cl.c = (cl.z * sp.ny + cl.y) * sp.nx + cl.x;
           const bool xfast = x0 >= sp.ix0 && min(x0 + 31, sp.nx - 1) < sp.ix0 + sp.ixn;
-          if (WALLS && sp.has_wall) {
-            step_cell<L, S, false, VARIANT, kPathShellRow, WALLS>(sb, db, sp, m.status, cl, valid, xfast);
-          } else {
-            long long* roff = s_roff[threadIdx.x >> 5];
-            shell_row_table<L>(roff, cl, sp);
-            step_cell<L, S, false, VARIANT, kPathShellTab, false>(sb, db, sp, m.status, cl, valid, xfast, roff);
-          }
+          long long* roff = s_roff[threadIdx.x >> 5];
+          uint32_t walled[4];
+          shell_row_table<L, WALLS>(roff, walled, cl, sp);
+          step_cell<L, S, false, VARIANT, kPathShellTab, WALLS>(sb, db, sp, m.status, cl, valid, xfast, roff, walled);
         }
       }
     }
@@ -1603,7 +1616,8 @@ __global__ void __launch_bounds__(kMomThreads) k_fields(const typename S::T* __r
   const int gid = blk * kMomThreads + threadIdx.x;
   const bool valid = gid < p.cells;
   const Cell cl = make_cell(valid ? gid : p.cells - 1, p);
-  const PullTab<L> tab(cl, p);
+  PullTab<L> tab(cl, p);
+  if constexpr (PULL && WALLS) tab.find_walls(cl, p);
   auto index = [&](auto I) -> long long {
     constexpr int i = decltype(I)::value;
     if constexpr (PULL) return tab.template index<i, WALLS>(cl, p);

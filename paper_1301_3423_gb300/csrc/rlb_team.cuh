@@ -144,7 +144,8 @@ __device__ __forceinline__ void team_tile(const typename S::T* src, typename S::
       for_slice(W, [&](auto I) { f[at(I).value] = load(base + p.off[decltype(I)::value]); });
     });
   } else {
-    const PullTab<L> tab(cl, p);
+    PullTab<L> tab(cl, p);
+    if constexpr (WALLS) tab.find_walls(cl, p);
     each_warp([&](auto W) {
       for_slice(W, [&](auto I) { f[at(I).value] = load(src + tab.template index<decltype(I)::value, WALLS>(cl, p)); });
     });
