@@ -66,11 +66,19 @@ cudaError_t init(const double* n, const double* Tf, const double* u, void* dst, 
 }
 
 cudaError_t convert_pops(void* pop, double* dbl, int i0, int i1, bool to_f64, const StepParams& p, cudaStream_t s) {
-  const int blocks = (p.cells + 127) / 128;
-  if (to_f64)
-    k_convert<L, S, true><<<blocks, 128, 0, s>>>((T*)pop, dbl, 0, i0, i1, p);
-  else
-    k_convert<L, S, false><<<blocks, 128, 0, s>>>((T*)pop, dbl, 0, i0, i1, p);
+  if constexpr (!std::is_same<S, StoreF16Dev>::value) {
+    // float and double populations are converted alike: one flat array of both (at most 2^38 elements,
+    // 1024 a block)
+    T* const q = (T*)pop + (long long)i0 * p.cells;
+    const long long n = (long long)(i1 - i0) * p.cells;
+    const unsigned blocks = (unsigned)((n + 4 * kConvertThreads - 1) / (4 * kConvertThreads));
+    if (to_f64) k_convert_flat<T, true><<<blocks, kConvertThreads, 0, s>>>(q, dbl, n);
+    else k_convert_flat<T, false><<<blocks, kConvertThreads, 0, s>>>(q, dbl, n);
+  } else {
+    const int blocks = (p.cells + 127) / 128;
+    if (to_f64) k_convert<L, S, true><<<blocks, 128, 0, s>>>((T*)pop, dbl, 0, i0, i1, p);
+    else k_convert<L, S, false><<<blocks, 128, 0, s>>>((T*)pop, dbl, 0, i0, i1, p);
+  }
   return cudaGetLastError();
 }
 
