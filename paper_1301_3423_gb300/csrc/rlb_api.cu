@@ -3,6 +3,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -349,6 +350,7 @@ extern "C" rlb_status rlb_create(const rlb_params* p, rlb_ctx** out) {
   c->fblocks = (c->cells + kMomThreads - 1) / kMomThreads;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
+  c->device = dev;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -479,6 +481,21 @@ static double* mapped_host(const double* p, size_t count) {
   return static_cast<double*>(a.devicePointer);
 }
 
+// True if array p[0 .. count) is memory of the context's device (both its ends are), so that a kernel
+// may write it; anything else goes through cudaMemcpyAsync, which checks the address.
+static bool on_this_device(const rlb_ctx* c, const double* p, size_t count) {
+  const double* const ends[2] = {p, p + (count - 1)};
+  for (const double* q : ends) {
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, q) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (a.type != cudaMemoryTypeDevice || a.device != c->device) return false;
+  }
+  return (reinterpret_cast<uintptr_t>(p) & 7) == 0;
+}
+
 extern "C" rlb_status rlb_init(rlb_ctx* c, const double* n, const double* T, const double* u, int on_device) {
   if (!c) return RLB_EINVAL;
   if (!n || !T || !u) return fail(c, RLB_EINVAL, "rlb_init: null field pointer");
@@ -606,13 +623,21 @@ extern "C" rlb_status rlb_moments(rlb_ctx* c, double* n, double* eps, double* U,
                       "fields kernel");
     if (st != RLB_OK) return st;
   } else if (on_device || (!n && !eps && !U)) {
-    st = check_launch(c, c->launch->fields(src, c->sp, staged, c->partial, c->status, pull, 0, c->fblocks, c->stream),
+    // the caller's device arrays are written in place (three copies of 48 bytes a cell less: 96 bytes a
+    // cell of traffic, and three launches where those count)
+    FieldOut out = staged;
+    const bool dn = n && on_this_device(c, n, cells), de = eps && on_this_device(c, eps, cells);
+    const bool dU = U && on_this_device(c, U, 4 * cells);
+    if (dn) out.f[0] = n;
+    if (de) out.f[1] = eps;
+    for (int k = 0; dU && k < 4; ++k) out.f[2 + k] = U + k * cells;
+    st = check_launch(c, c->launch->fields(src, c->sp, out, c->partial, c->status, pull, 0, c->fblocks, c->stream),
                       "fields kernel");
     if (st != RLB_OK) return st;
     const size_t cb = cells * sizeof(double);
-    if (n) RLB_CUDA(c, cudaMemcpyAsync(n, c->fields, cb, cudaMemcpyDeviceToDevice, c->stream));
-    if (eps) RLB_CUDA(c, cudaMemcpyAsync(eps, c->fields + cells, cb, cudaMemcpyDeviceToDevice, c->stream));
-    if (U) RLB_CUDA(c, cudaMemcpyAsync(U, c->fields + 2 * cells, 4 * cb, cudaMemcpyDeviceToDevice, c->stream));
+    if (n && !dn) RLB_CUDA(c, cudaMemcpyAsync(n, c->fields, cb, cudaMemcpyDeviceToDevice, c->stream));
+    if (eps && !de) RLB_CUDA(c, cudaMemcpyAsync(eps, c->fields + cells, cb, cudaMemcpyDeviceToDevice, c->stream));
+    if (U && !dU) RLB_CUDA(c, cudaMemcpyAsync(U, c->fields + 2 * cells, 4 * cb, cudaMemcpyDeviceToDevice, c->stream));
   } else {
     // host outputs: the fields of chunk j are copied out on the copy stream while the fields kernel
     // of chunk j + 1 runs on the context's stream
