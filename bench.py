@@ -152,6 +152,8 @@ def step_kernel_name(variant):
     """The kernels one time step of float storage launches with this variant."""
     from paper_1301_3423_gb300.rlb import VARIANT_NAMES
     name = VARIANT_NAMES[variant] if 0 <= variant < len(VARIANT_NAMES) else str(variant)
+    if name.startswith("team"):
+        return "k_step_team<Quad3, StoreF32> (%s)" % name
     if variant >= 4:
         return "k_step_pipe<Quad3, StoreF32> (%s; one launch per step)" % name
     return "k_step_interior + k_step_shell_rows <Quad3, StoreF32, variant %d> (%s)" % (variant, name)

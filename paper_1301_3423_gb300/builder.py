@@ -7,6 +7,7 @@ the flags are unchanged (content hash)."""
 import concurrent.futures as cf
 import hashlib
 import os
+import re
 import shutil
 import subprocess
 import sys
@@ -98,8 +99,12 @@ def build(force=False, verbose=False):
         jobs.append((obj, [nvcc] + NVCC_FLAGS + inc + ["-DRLB_INST_ORDER=%d" % o, "-DRLB_INST_STORAGE=%d" % s,
                                                           "-DRLB_INST_TX=%d" % tx, "-DRLB_INST_ROWS=%d" % rows, "-c",
                                                           os.path.join(CSRC, "rlb_inst_pipe.cu"), "-o", obj]))
-    # longest units first so the parallel build ends sooner
-    jobs = jobs[:1] + sorted(jobs[1:], key=lambda j: ("_v" not in j[0], "_s0" in j[0]))
+    # longest units first so the parallel build ends sooner (the pipelined ones, then the step variants)
+    def order(job):
+        name = os.path.basename(job[0])
+        return (re.search(r"_[xr]\d+\.o$", name) is None, "_v" not in name, "_s0" in name)
+
+    jobs = jobs[:1] + sorted(jobs[1:], key=order)
     jobs[0][1].extend(["-o", jobs[0][0]])
     logs = []
     with cf.ThreadPoolExecutor(max_workers=min(len(jobs), max(os.cpu_count() or 4, 4))) as ex:

@@ -29,9 +29,9 @@ struct PipeConfig {
 // always refers to the phase it means.  With as many stages as groups each group refills its one
 // stage while the other groups compute.
 // A bulk copy takes some 45 clocks of an SM whatever its length (measured: 39 to 47 M copies/s and SM
-// from 132 to 528 bytes each), so the wide shapes copy the most per instruction that their stages
-// allow, and eight producer warps keep the copies going while four consumers' worth of registers would
-// only wait (256^3 float: 4 producers 3.03 ms, 8 2.91, 12 with 80 registers a thread 3.09).
+// of 272 to 528 bytes each), so the wide shapes copy the most per instruction that their stages allow,
+// and the default shapes have eight producer warps to keep copies under way (256^3 float: 4 producers
+// 3.03 ms a step, 8 2.91, 12 with 80 registers a thread 3.09; 96^3 0.183, 0.166, 0.182).
 constexpr PipeConfig kPipeConfigs[] = {
     {128, 8, 1, 8, 0, 1}, {128, 8, 1, 4, 0, 1},  {64, 8, 1, 8, 0, 1},  {64, 4, 1, 4, 0, 1},
     {128, 8, 1, 6, 0, 1}, {64, 8, 1, 4, 0, 1},   {128, 4, 1, 4, 0, 1}, {64, 2, 1, 4, 0, 1},

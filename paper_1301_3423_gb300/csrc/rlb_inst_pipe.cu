@@ -73,10 +73,8 @@ cudaError_t RLB_PIPE_FN(pipe_batch, RLB_INST_TX)(const BatchMember* m, const int
     return cudaErrorInvalidValue;
   }
   if constexpr (kOneWarp && kWide) return cudaErrorInvalidValue;
-  else {
-  if (walls) return launch_pipe_batch<true, false>(m, tm, launch, pp, timeout, grid, threads, smem, s);
-  return launch_pipe_batch<false, false>(m, tm, launch, pp, timeout, grid, threads, smem, s);
-  }
+  else if (walls) return launch_pipe_batch<true, false>(m, tm, launch, pp, timeout, grid, threads, smem, s);
+  else return launch_pipe_batch<false, false>(m, tm, launch, pp, timeout, grid, threads, smem, s);
 }
 
 // One time step of the whole lattice in one launch, compiled with the bounce-back patch only for
@@ -92,9 +90,7 @@ cudaError_t RLB_PIPE_FN(pipe, RLB_INST_TX)(const void* src, void* dst, const Ste
     return cudaErrorInvalidValue;
   }
   if constexpr (kOneWarp && kWide) return cudaErrorInvalidValue;
-  else {
-  if (p.has_wall) return launch_pipe<true, false>(src, dst, p, pp, status, grid, threads, smem, s);
-  return launch_pipe<false, false>(src, dst, p, pp, status, grid, threads, smem, s);
-  }
+  else if (p.has_wall) return launch_pipe<true, false>(src, dst, p, pp, status, grid, threads, smem, s);
+  else return launch_pipe<false, false>(src, dst, p, pp, status, grid, threads, smem, s);
 }
 }  // namespace rlb

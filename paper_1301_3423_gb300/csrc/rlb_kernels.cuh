@@ -1,6 +1,7 @@
 // Kernels of the relativistic lattice Boltzmann step (arXiv:1301.3423) for sm_103a.
 //
-// One thread owns one cell.  A step (Eq. (rlb:disc)) is a single fused pass per cell:
+// A step (Eq. (rlb:disc)) is a single fused pass per cell, by one thread per cell in the kernels here
+// (rlb_pipe.cuh stages the pull in shared memory, rlb_team.cuh splits a cell between four warps):
 //   pull    f~_i(x) = f_i(x - v_i)                     one read per population
 //   moments N^mu, T^{mu nu} over mirror pairs         (Sec. II.D)
 //   Landau  T^{ab} U_b = eps U^a, n = U.N, T = eps/(3n) (Eq. (eigenproblem))
@@ -1598,7 +1599,9 @@ static __device__ __noinline__ Landau<double> landau_readout_fp64(const Mom<doub
 // ---------------------------------------------------------------------------------------------
 // fields and conserved densities of one time level.  Double storage: double moments and Landau solve.
 // Float storages: float moments (moments_pd), the step's Landau policy, and one update of a float
-// frame in float-float (frame_update).
+// frame in float-float (frame_update).  128^3 float: 357 us, 0.49 of the copy bandwidth, bound by
+// instruction issue; 767 us with the update in double and every coordinate of every pull wrapped by
+// itself.  Double: 96^3 876 us against 2563 (integer sums, corrected frame).
 //   PULL = true : the pre-collision populations pulled from the previous state
 //   PULL = false: the stored populations of each cell
 // out.f[k][cell], k = n, eps, U0, U1, U2, U3; partial[block][5] = block sums of
@@ -1810,8 +1813,9 @@ __global__ void __launch_bounds__(128) k_init(const double* __restrict__ n, cons
     // (compensated; the even part a + c t^2 and the odd part t (b + d t^2) shared by +v and -v), the
     // others in float: every population ends within float rounding of the double evaluation.  The
     // inputs are normalised in double (some 40 operations a cell, which the 1/64-rate pipe does
-    // beside the float work); the coefficients, 110 double operations a cell and the bound of this
-    // kernel while they were double, are float-float.
+    // beside the float work: 40 % busy); the coefficients, 110 double operations a cell and the bound
+    // of this kernel while they were double, are float-float.  128^3 float: 364 us, 876 before; bound
+    // by float issue (4640 warp instructions per 32 cells, issue slots 67 %, FMA pipe 63 % used).
     const LevCoef<L, FF> e = level_coef_ff<L>(ff_from(nn), ff_from(T), ff_from(fma(T, g, -1.0)));
     // U / R times 1 .. 6 per axis: t = v.U / R is then a sum of at most three of them
     FF m[3][7];

@@ -2,6 +2,10 @@
 // (TMA) engine, with warp-specialised producer and consumer warps (sm_90+ PTX: mbarrier,
 // cp.async.bulk).
 //
+// A bulk copy takes an SM about 45 clocks whatever its length (39 to 47 M copies/s and SM measured from
+// 272 to 528 bytes each); with the 1024 bytes a float cell update moves, that is what bounds the kernel
+// once enough producers issue them, at 0.9 of the copy bandwidth for float rows of 128 cells and more.
+//
 // A tile is one 64- or 128-cell segment of a lattice row (fixed y, z; x0 a multiple of the tile
 // width TX).  For every population i the cells x0 .. x0 + TX - 1 pull from the row
 // (y - vy_i, z - vz_i) at x - vx_i, i.e. from one contiguous run of the source plane.  The
@@ -17,7 +21,7 @@
 // offset i * BX + r_i + x of the stage (r_i = -vx_i mod the copy granule), twice: once for the
 // moments and once for the collision, whose result goes straight to global memory with one
 // coalesced store per population.  The populations never sit in registers as a whole, so a
-// consumer needs at most 128 registers instead of Q + ~40, and the loads that feed a tile are
+// consumer needs 96 registers (128 double) instead of Q + ~40, and the loads that feed a tile are
 // issued by one producer lane per population instead of 32 lanes each computing an address.
 //
 // Row tiles (ROWS): on an x-periodic lattice with rows of nx <= TX cells a tile is G = TX / nx
@@ -37,7 +41,7 @@
 // their copies have landed, empty[s][c] when every consumer warp of that tile has read the chunk for
 // the last time.  Moments and collision go through the chunks in order, so the next tile's first chunk
 // is on its way while the last is still being collided, and its moments start before its last chunk
-// has landed.  (256^3 float step, 8 producers: 2.82 ms in four chunks, 2.91 in one; row tiles, whose
+// has landed.  (256^3 float step, 8 producers: 2.85 ms in four chunks, 2.91 in one; row tiles, whose
 // tiles refill with one copy per population: 128^3 0.377 ms in four, 0.352 in one.)  Every wait is
 // bounded (kPipeWaitNs); a wait that runs out counts in status[kStatusTimeout], and the producer
 // then waits (bounded) for the copies it has in flight before it returns.
@@ -308,51 +312,51 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
         __syncwarp();
         if (!tr.active) continue;
         for (int j = lane; j < mine; j += 32) {
-        const int i = c * CH + first + j * share;
-        const char4 v = sv[i];
-        const long long plane = (long long)i * p.cells;
-        T* const d = st + i * BX;
-        if constexpr (ROWS) {
-          // each run of consecutive source rows with one copy of whole rows
-          int r = 0, yr = y, zr = z;
-          long long run0 = 0, next = -1;
-          int runlen = 0;
-          for (; r < gt; ++r) {
-            const long long sr = (long long)pipe_src_row(zr - v.z, p.nz, p.bc[2]) * p.ny +
-                                 pipe_src_row(yr - v.y, p.ny, p.bc[1]);
-            if (sr != next) {
-              if (runlen > 0) copy(d + (r - runlen) * p.nx, plane + run0 * p.nx, runlen * p.nx, bar);
-              run0 = sr;
-              runlen = 0;
+          const int i = c * CH + first + j * share;
+          const char4 v = sv[i];
+          const long long plane = (long long)i * p.cells;
+          T* const d = st + i * BX;
+          if constexpr (ROWS) {
+            // each run of consecutive source rows with one copy of whole rows
+            int r = 0, yr = y, zr = z;
+            long long run0 = 0, next = -1;
+            int runlen = 0;
+            for (; r < gt; ++r) {
+              const long long sr = (long long)pipe_src_row(zr - v.z, p.nz, p.bc[2]) * p.ny +
+                                       pipe_src_row(yr - v.y, p.ny, p.bc[1]);
+              if (sr != next) {
+                if (runlen > 0) copy(d + (r - runlen) * p.nx, plane + run0 * p.nx, runlen * p.nx, bar);
+                run0 = sr;
+                runlen = 0;
+              }
+              ++runlen;
+              next = sr + 1;
+              if (++yr == p.ny) {
+                yr = 0;
+                ++zr;
+              }
             }
-            ++runlen;
-            next = sr + 1;
-            if (++yr == p.ny) {
-              yr = 0;
-              ++zr;
+            copy(d + (r - runlen) * p.nx, plane + run0 * p.nx, runlen * p.nx, bar);
+          } else {
+            const long long row0 =
+                plane + ((long long)pipe_src_row(z - v.z, p.nz, p.bc[2]) * p.ny + pipe_src_row(y - v.y, p.ny, p.bc[1])) * p.nx;
+            const int xs = (x0 - v.x) & ~(AL - 1);  // round down to a granule (two's complement: floor)
+            if (xperiodic && (xs < 0 || xs + BX > p.nx)) {
+              // split [xs, xs + BX) at multiples of nx; each piece is whole granules of one period
+              int a = xs;
+              const int e = xs + BX;
+              while (a < e) {
+                const int per = (a >= 0) ? a / p.nx : -((-a + p.nx - 1) / p.nx);
+                const int pe = min(e, (per + 1) * p.nx);
+                copy(d + (a - xs), row0 + (a - per * p.nx), pe - a, bar);
+                a = pe;
+              }
+            } else {
+              // x beyond the ends reads neighbouring memory (guard bytes around every buffer); the
+              // consumer patches those cells
+              copy(d, row0 + xs, BX, bar);
             }
           }
-          copy(d + (r - runlen) * p.nx, plane + run0 * p.nx, runlen * p.nx, bar);
-        } else {
-        const long long row0 =
-            plane + ((long long)pipe_src_row(z - v.z, p.nz, p.bc[2]) * p.ny + pipe_src_row(y - v.y, p.ny, p.bc[1])) * p.nx;
-        const int xs = (x0 - v.x) & ~(AL - 1);  // round down to a granule (two's complement: floor)
-        if (xperiodic && (xs < 0 || xs + BX > p.nx)) {
-          // split [xs, xs + BX) at multiples of nx; each piece is whole granules of one period
-          int a = xs;
-          const int e = xs + BX;
-          while (a < e) {
-            const int per = (a >= 0) ? a / p.nx : -((-a + p.nx - 1) / p.nx);
-            const int pe = min(e, (per + 1) * p.nx);
-            copy(d + (a - xs), row0 + (a - per * p.nx), pe - a, bar);
-            a = pe;
-          }
-        } else {
-          // x beyond the ends reads neighbouring memory (guard bytes around every buffer); the
-          // consumer patches those cells
-          copy(d, row0 + xs, BX, bar);
-        }
-        }
         }
       }
     }
