@@ -239,7 +239,12 @@ static int default_variant(const rlb_ctx* c) {
     if (rows >= 0) return rows;
     const int seg = 15;
     PipeLayout lay;
+    // An x that is not periodic is patched in shared memory population by population in the first and
+    // last segment of each row, a chain of loads that the register kernels do not have: a job of such
+    // rows ran at 0.6 ns a cell update here, 0.33 to 0.35 on the register kernels (151 x 93 x 70).  So
+    // only where those two segments are less than half of a row.
     if (pipe_layout(seg, c->q, (int)c->elem, c->smem_per_sm, c->smem_optin, &lay) &&
+        (c->sp.bc[0] == kPeriodic || c->sp.nx > 4 * lay.tx) &&
         pipe_fits(c->sp.nx, lay.tx, (int)c->elem, fill_eighths(lay, (int)c->elem)) && variant_available(c, seg))
       return seg;
   }
