@@ -176,10 +176,12 @@ rlb_status rlb_set_populations(rlb_ctx* ctx, const double* f, int on_device);
  *         only for lattices with a periodic x of at most 128 cells (and at least the stencil's
  *         x reach), nx again a multiple of 16 bytes' worth of populations.
  *   15..18 row segments (15, 17) and row tiles (16, 18) in three consumer groups of four warps
- *         per block, 8 (15, 16) or 2 (17, 18) producer warps; float storage relaxes each cell in
- *         one warp here instead of two, and row segments are refilled in four chunks.
+ *         per block, 8 (15, 16; 4 with double storage) or 2 (17, 18) producer warps; float storage
+ *         relaxes each cell in one warp here instead of two, and row segments are refilled in four
+ *         chunks.  Double storage has them at the second order, whose stages fit.
  *   19    96-cell row tiles (rows of at most 96 cells; 96, 48 and 32 fill them), four consumer
- *         groups of three warps, one warp per float cell.
+ *         groups of three warps, one warp per float cell, 8 producer warps (double storage: 4, and
+ *         at the second order only).
  *   20    the team kernel: the four warps of a block share 32 consecutive cells, a quarter of the
  *         populations each; every storage and lattice.  On small lattices (the default for those
  *         whose rows do not suit the pipelined kernel) rlb_step runs up to 64 steps in one

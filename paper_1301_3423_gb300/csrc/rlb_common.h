@@ -10,15 +10,16 @@ constexpr int kDefaultStepVariant = 0;  // step-kernel variant before autotuning
 
 // Step-kernel variants.  0..3: one cell per thread with all populations in registers (float
 // storages; double storage has variant 0 only, which reads its populations twice).  4 and up: the
-// pipelined kernel (k_step_pipe) in the shapes of kPipeConfigs, for every storage, on lattices whose
-// rows start on 16-byte boundaries.
+// pipelined kernel (k_step_pipe) in the shapes of kPipeConfigs, for the storages whose stages fit a block
+// (pipe_layout), on lattices whose rows start on 16-byte boundaries.
 constexpr int kNumRegVariants = 4;
 struct PipeConfig {
-  int tx;           // tile width in cells (64 or 128; 96 for row tiles)
+  int tx;           // tile width in cells (64 or 128; row tiles 96, 128, 160, 192 or 256)
   int cons_warps;   // consumer warps per block: TX / 32 per tile, twice that with float storage
                     // (two warps per cell); a multiple of the warps per tile
   int ctas_per_sm;  // resident blocks per SM (the shared memory is split between them)
-  int producers;    // producer warps per block (each copies every producers-th population of every tile)
+  int producers;    // producer warps per block, together on every tile; double storage, whose blocks have
+                    // fewer warps (pipe_max_warps), takes as many of them as fit (pipe_layout)
   int rows;         // 0: a tile is a TX-cell segment of one row; 1: a tile is TX / nx whole rows of
                     // an x-periodic lattice with nx <= TX ("row tiles", one copy per population)
   int split;        // float storage: 1 = two warps per cell (each half the populations), 0 = one;

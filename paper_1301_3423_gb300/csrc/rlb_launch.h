@@ -109,16 +109,18 @@ inline bool pipe_layout(int v, int q, int elem, int smem_per_sm, int smem_optin,
   const bool split = elem == 4 && cf.split;  // float storage: two consumer warps per cell
   const int wpt = cf.tx / 32 * (split ? 2 : 1);
   const int groups = cf.cons_warps / wpt;
-  if (groups < 1 || cf.cons_warps % wpt != 0 || cf.producers < 1 || cf.producers > q) return false;
-  if (cf.producers > kPipeMaxProducerWarps || cf.cons_warps > kPipeMaxConsumerWarps ||
-      cf.cons_warps + cf.producers > pipe_max_warps(elem))
-    return false;
+  // The producers that the kernel's warps leave room for: twelve consumer warps leave double storage, whose
+  // cells need 128 registers a thread, four of the eight that float and half storage have.
+  const int room = pipe_max_warps(elem) - cf.cons_warps;
+  const int producers = cf.producers < room ? cf.producers : room;
+  if (groups < 1 || cf.cons_warps % wpt != 0 || producers < 1 || producers > q) return false;
+  if (producers > kPipeMaxProducerWarps || cf.cons_warps > kPipeMaxConsumerWarps) return false;
   const long long xchg = split ? (long long)cf.cons_warps / 2 * kPipeXchgBytesPerPair : 0;
   long long fit = (budget - kPipeHeaderBytes - xchg) / stage;
   if (fit > kPipeMaxStages) fit = kPipeMaxStages;
   const int nstage = (int)(fit / groups * groups);
   if (nstage < groups || nstage < 2) return false;
-  if (out) *out = PipeLayout{cf.tx, nstage, groups, cf.producers, (cf.cons_warps + cf.producers) * 32,
+  if (out) *out = PipeLayout{cf.tx, nstage, groups, producers, (cf.cons_warps + producers) * 32,
                              (int)(kPipeHeaderBytes + nstage * stage + xchg), cf.ctas_per_sm, cf.rows, split};
   return true;
 }
