@@ -82,39 +82,40 @@ cudaError_t convert_pops(void* pop, double* dbl, int i0, int i1, bool to_f64, co
   return cudaGetLastError();
 }
 
+// The units that exist (see pipe_built): double storage of the third order has 64-cell segments only.
 cudaError_t pipe_step(const void* src, void* dst, const StepParams& p, const PipeParams& pp, int* status, int tx,
                       int rows, int split, int grid, int threads, int smem, cudaStream_t s) {
-  if (rows) {
-    if (tx == 96) return RLB_RFN(pipe, 96)(src, dst, p, pp, status, split, grid, threads, smem, s);
+#if RLB_PIPE128
+  if (rows && tx == 96) return RLB_RFN(pipe, 96)(src, dst, p, pp, status, split, grid, threads, smem, s);
+  if (rows && tx == 128) return RLB_RFN(pipe, 128)(src, dst, p, pp, status, split, grid, threads, smem, s);
+  if (!rows && tx == 128) return RLB_PFN(pipe, 128)(src, dst, p, pp, status, split, grid, threads, smem, s);
+#endif
 #if RLB_WIDE
-    if (tx == 160) return RLB_RFN(pipe, 160)(src, dst, p, pp, status, split, grid, threads, smem, s);
-    if (tx == 192) return RLB_RFN(pipe, 192)(src, dst, p, pp, status, split, grid, threads, smem, s);
+  if (rows && tx == 160) return RLB_RFN(pipe, 160)(src, dst, p, pp, status, split, grid, threads, smem, s);
+  if (rows && tx == 192) return RLB_RFN(pipe, 192)(src, dst, p, pp, status, split, grid, threads, smem, s);
 #endif
 #if RLB_WIDE256
-    if (tx == 256) return RLB_RFN(pipe, 256)(src, dst, p, pp, status, split, grid, threads, smem, s);
+  if (rows && tx == 256) return RLB_RFN(pipe, 256)(src, dst, p, pp, status, split, grid, threads, smem, s);
 #endif
-    if (tx != 128) return cudaErrorInvalidValue;
-    return RLB_RFN(pipe, 128)(src, dst, p, pp, status, split, grid, threads, smem, s);
-  }
-  if (tx == 128) return RLB_PFN(pipe, 128)(src, dst, p, pp, status, split, grid, threads, smem, s);
+  if (rows || tx != 64) return cudaErrorInvalidValue;
   return RLB_PFN(pipe, 64)(src, dst, p, pp, status, split, grid, threads, smem, s);
 }
 
 cudaError_t pipe_batch_step(const BatchMember* m, const int* tm, int launch, const PipeParams& pp, int* timeout, int tx,
                             int rows, int split, int walls, int grid, int threads, int smem, cudaStream_t s) {
-  if (rows) {
-    if (tx == 96) return RLB_RFN(pipe_batch, 96)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
+#if RLB_PIPE128
+  if (rows && tx == 96) return RLB_RFN(pipe_batch, 96)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
+  if (rows && tx == 128) return RLB_RFN(pipe_batch, 128)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
+  if (!rows && tx == 128) return RLB_PFN(pipe_batch, 128)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
+#endif
 #if RLB_WIDE
-    if (tx == 160) return RLB_RFN(pipe_batch, 160)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
-    if (tx == 192) return RLB_RFN(pipe_batch, 192)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
+  if (rows && tx == 160) return RLB_RFN(pipe_batch, 160)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
+  if (rows && tx == 192) return RLB_RFN(pipe_batch, 192)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
 #endif
 #if RLB_WIDE256
-    if (tx == 256) return RLB_RFN(pipe_batch, 256)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
+  if (rows && tx == 256) return RLB_RFN(pipe_batch, 256)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
 #endif
-    if (tx != 128) return cudaErrorInvalidValue;
-    return RLB_RFN(pipe_batch, 128)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
-  }
-  if (tx == 128) return RLB_PFN(pipe_batch, 128)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
+  if (rows || tx != 64) return cudaErrorInvalidValue;
   return RLB_PFN(pipe_batch, 64)(m, tm, launch, pp, timeout, split, walls, grid, threads, smem, s);
 }
 

@@ -56,7 +56,7 @@ cudaError_t launch_pipe_batch(const BatchMember* m, const int* tm, int launch, c
 
 // One warp per float cell exists for float storage from 96-cell tiles up.
 constexpr bool kOneWarp = std::is_same<S, StoreF32>::value && RLB_INST_TX >= 96;
-constexpr bool kWide = RLB_INST_TX > 128;  // one warp per float cell only
+constexpr bool kOneWarpOnly = kOneWarp && RLB_INST_TX != 128;  // no shape of these widths has two
 }  // namespace
 
 // One time step of every active batch member on the pipelined kernel (walls: some member has
@@ -72,7 +72,7 @@ cudaError_t RLB_PIPE_FN(pipe_batch, RLB_INST_TX)(const BatchMember* m, const int
   } else if (!split && std::is_same<S, StoreF32>::value) {
     return cudaErrorInvalidValue;
   }
-  if constexpr (kOneWarp && kWide) return cudaErrorInvalidValue;
+  if constexpr (kOneWarpOnly) return cudaErrorInvalidValue;
   else if (walls) return launch_pipe_batch<true, false>(m, tm, launch, pp, timeout, grid, threads, smem, s);
   else return launch_pipe_batch<false, false>(m, tm, launch, pp, timeout, grid, threads, smem, s);
 }
@@ -89,7 +89,7 @@ cudaError_t RLB_PIPE_FN(pipe, RLB_INST_TX)(const void* src, void* dst, const Ste
   } else if (!split && std::is_same<S, StoreF32>::value) {
     return cudaErrorInvalidValue;
   }
-  if constexpr (kOneWarp && kWide) return cudaErrorInvalidValue;
+  if constexpr (kOneWarpOnly) return cudaErrorInvalidValue;
   else if (p.has_wall) return launch_pipe<true, false>(src, dst, p, pp, status, grid, threads, smem, s);
   else return launch_pipe<false, false>(src, dst, p, pp, status, grid, threads, smem, s);
 }

@@ -55,6 +55,7 @@ RLB_DECLARE_PIPE(128)
 #undef RLB_DECLARE_PIPE
 // ... and with row tiles (RLB_INST_ROWS = 1), tile widths 128, 96 and the wide ones that are built
 // (pipe_built).
+#define RLB_PIPE128 (RLB_INST_STORAGE != 0 || RLB_INST_ORDER == 2)  // 96- and 128-cell tiles
 #define RLB_WIDE (RLB_INST_STORAGE != 0)
 #define RLB_WIDE256 (RLB_INST_STORAGE == 2 || (RLB_INST_STORAGE == 1 && RLB_INST_ORDER == 2))
 #define RLB_RFN(fn, tx) RLB_CAT7(fn, _o, RLB_INST_ORDER, _s, RLB_INST_STORAGE, _r, tx)

@@ -93,8 +93,10 @@ inline long long pipe_tile_count(int nx, int ny, int nz, int tx, int rows) {
 }
 
 // Tile widths above 128 are built for the float storages, 256 only where two stages of it fit (half
-// storage, and the second order's 66 float populations).
+// storage, and the second order's 66 float populations); of double storage's third order only the
+// 64-cell tiles (a stage of 96 cells is 100 KB and the shape's four consumer groups want one each).
 constexpr bool pipe_built(int tx, int q, int elem) {
+  if (q * elem == 128 * 8) return tx == 64;
   return tx <= 128 || (elem < 8 && (tx < 256 || q * elem < 128 * 4));
 }
 

@@ -62,3 +62,19 @@ def test_shapes_exist(layout, order, storage):
         assert lay["threads"] <= 32 * layout.max_warps(storage)
         assert lay["nstage"] >= 2 and lay["nstage"] % lay["groups"] == 0 and lay["smem"] <= SMEM_PER_BLOCK
         assert 1 <= lay["producers"] <= lay["threads"] // 32 - 1
+
+
+@pytest.mark.parametrize("order,storage", sorted(SHAPES))
+def test_units_built_are_the_ones_a_shape_needs(layout, order, storage):
+    needed = {(lay["tx"], lay["rows"]) for lay in (layout(v, order, storage) for v in range(24)) if lay}
+    s = list(ELEM).index(storage)
+    assert sorted(needed) == sorted((tx, rows) for o, t, tx, rows in builder.PIPE_UNITS if (o, t) == (order, s))
+
+
+def test_built_tree_is_small():
+    """The library's folder travels with the tree: no objects are left in it, and it stays far below the
+    few hundred megabytes that a copy of the tree may have."""
+    builder.build()
+    files = [os.path.join(d, f) for d, _, fs in os.walk(builder.BUILD) for f in fs]
+    assert not [f for f in files if f.endswith(".o")]
+    assert sum(os.path.getsize(f) for f in files) < 100e6
