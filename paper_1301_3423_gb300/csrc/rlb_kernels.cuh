@@ -413,26 +413,40 @@ struct Slices {
       if (slice_of(k) == s && (l < 0 || L::LEV[2 * k] == l) && j-- == 0) return 2 * k;
     return -1;
   }
-  __host__ __device__ static constexpr int sum(int s, int l, int a, int b) {  // of v_a v_b
-    int r = 0;
-    for (int k = 0; k < PAIRS; ++k) {
-      const int v[3] = {L::VX[2 * k], L::VY[2 * k], L::VZ[2 * k]};
-      if (slice_of(k) == s && L::LEV[2 * k] == l) r += v[a] * v[b];
-    }
-    return r;
+  // the largest sum of |weights| (1, v_a, v_a v_b) over the populations of slice s and level l
+  __host__ __device__ static constexpr int weight(int s, int l) {
+    int most = 2 * count(s, l);
+    for (int a = 0; a < 3; ++a)
+      for (int b = 0; b <= 3; ++b) {
+        int r = 0;
+        for (int k = 0; k < PAIRS; ++k) {
+          const int v[4] = {L::VX[2 * k], L::VY[2 * k], L::VZ[2 * k], 1}, w = v[a] * v[b];
+          if (slice_of(k) == s && L::LEV[2 * k] == l) r += 2 * (w < 0 ? -w : w);
+        }
+        most = r > most ? r : most;
+      }
+    return most;
+  }
+  // bits a population may have so that every sum stays below 2^63
+  __host__ __device__ static constexpr int bits(int s, int l) {
+    int n = 63;
+    for (int w = weight(s, l); w > 1; w = (w + 1) / 2) --n;
+    return n;
   }
 };
 
 // Moments of double populations, summed in 64-bit integers.  GB300's double pipe takes 19 clocks an
 // SM for a warp instruction (measured; 64 for a lone warp) and bounds the double step; its integer
-// pipe is some 40 times wider.  Per slice and energy level the populations are put on a common grid
-// of 2^-50 to 2^-51 of the largest of them (adding 1.5 2^k leaves the grid value in the low bits of
-// the sum), and the sums over v with the integer weights 1, v_a, v_a v_b are exact integers:
-// |v_a v_b| sums to at most 2^11 over the populations, so 51 + 11 bits and the sign fit.  Then 9 sums
-// return to double and take p0 and p0^2.  The grid is per level, so the rare high levels, which p0^2
-// weights most, are rounded by their own size: the moments' error is below that of adding the 128
-// terms in double (fields of a 96^3 run against 64-bit references: 4.2e-16 here, 4.6e-16 before).
-// Double operations a cell: 128 adds, 63 conversions, 140 more; 960 when the sums were double.
+// pipe is some 40 times wider.  Per slice and energy level the populations are converted to integers of
+// a common grid, 2^-53 to 2^-58 of the power of two above the largest of them, as fine as 63-bit sums allow
+// (Slices::bits): the scale goes into the exponent as an integer and the conversion takes 16 clocks.  The
+// sums over v with the integer weights 1, v_a, v_a v_b are exact; 9 of them return to double and take p0
+// and p0^2.  The grid is per level, so the rare high levels, which p0^2 weights most, are rounded by
+// their own size.  The moments' error is below that of adding the 128 terms in double up to a Lorentz
+// factor of 4 (third order, r.m.s. of T^00: 4.4e-17 against 8.0e-17 at rest, 7.2e-17 against 1.4e-16 at
+// 2).  A grid of 2^-51 from adding 1.5 2^k was two to three times worse from 1.5 on and saved 1 % (96^3,
+// ten steps: 25.4 ms against 25.7).
+// Double-pipe instructions a cell: 128 conversions there, 63 back, 140 more; 960 when the sums were double.
 // Populations that are not finite (or beyond 2^1021, whose moments overflow) give NaN moments.
 // Slice SL's part, before the factors 1 / R and 1 / R^2 (finish_fixed).
 template <class L, int SL, class Get>
@@ -448,6 +462,8 @@ __device__ __forceinline__ Mom<double> moments_fixed_slice(Get&& get) {
     constexpr int l = decltype(K)::value;
     constexpr int n = G::count(SL, l);
     if constexpr (n > 0) {
+      constexpr int BITS = G::bits(SL, l);
+      static_assert(BITS >= 53 && BITS <= 62, "every double below 2^BITS rounds to an integer below it");
       double f[2 * n];
       unsigned top = 0;
       static_for<n>([&](auto J) {
@@ -459,15 +475,18 @@ __device__ __forceinline__ Mom<double> moments_fixed_slice(Get&& get) {
       });
       const int e = max((int)(top >> 20), 64);  // |f| < 2^(e - 1022)
       finite = finite && e < 2045;
-      const double C = __hiloint2double(((e + 2) << 20) | 0x80000, 0);  // 1.5 2^(e - 1021)
-      const u64 Cb = (u64)__double_as_longlong(C);
-      // sums of the raw bits; each carries a known multiple of those of C, removed below (modulo 2^64)
+      // f 2^(BITS + 1022 - e) as an integer below 2^BITS.  Where the scaled exponent would be negative or
+      // 0, the number is less than 1/2 (and stays so when 0 or a subnormal gets an exponent).
+      const int shift = (BITS + 1022 - e) * (1 << 20);
+      auto grid = [&](double x) -> u64 {
+        const int h = __double2hiint(x), t = max((h & 0x7fffffff) + shift, 0);
+        return (u64)__double2ll_rn(__hiloint2double(t | (h & (int)0x80000000u), __double2loint(x)));
+      };
       u64 s0 = 0, sxx = 0, syy = 0, sxy = 0, sxz = 0, syz = 0, sx = 0, sy = 0, sz = 0;
       static_for<n>([&](auto J) {
         constexpr int j = decltype(J)::value, i = G::pair(SL, l, j);
         constexpr int vx = L::VX[i], vy = L::VY[i], vz = L::VZ[i];
-        const u64 a = (u64)__double_as_longlong(__dadd_rn(f[2 * j], C));
-        const u64 b = (u64)__double_as_longlong(__dadd_rn(f[2 * j + 1], C));
+        const u64 a = grid(f[2 * j]), b = grid(f[2 * j + 1]);
         const u64 sp = a + b, sm = a - b;
         s0 += sp;
         if constexpr (vx != 0) sxx += (u64)(long long)(vx * vx) * sp, sx += (u64)(long long)vx * sm;
@@ -477,10 +496,10 @@ __device__ __forceinline__ Mom<double> moments_fixed_slice(Get&& get) {
         if constexpr (vx * vz != 0) sxz += (u64)(long long)(vx * vz) * sp;
         if constexpr (vy * vz != 0) syz += (u64)(long long)(vy * vz) * sp;
       });
-      auto even = [&](u64 s, int w) { return (double)(long long)(s - (u64)(2ll * w) * Cb); };
-      const double g = __hiloint2double((e - 50) << 20, 0);  // the grid, 2^(e - 1073)
+      auto dbl = [](u64 s) { return (double)(long long)s; };
+      const double g = __hiloint2double((e + 1 - BITS) << 20, 0);  // the grid, 2^(e - 1022 - BITS)
       const double p1 = L::P0[l] * g, p2 = L::P0[l] * L::P0[l] * g;
-      const double d0 = even(s0, n), dx = (double)(long long)sx, dy = (double)(long long)sy, dz = (double)(long long)sz;
+      const double d0 = dbl(s0), dx = dbl(sx), dy = dbl(sy), dz = dbl(sz);
       m.N0 = fma(p1, d0, m.N0);
       m.Nx = fma(p1, dx, m.Nx);
       m.Ny = fma(p1, dy, m.Ny);
@@ -489,11 +508,11 @@ __device__ __forceinline__ Mom<double> moments_fixed_slice(Get&& get) {
       m.T0x = fma(p2, dx, m.T0x);
       m.T0y = fma(p2, dy, m.T0y);
       m.T0z = fma(p2, dz, m.T0z);
-      m.Txx = fma(p2, even(sxx, ic<G::sum(SL, l, 0, 0)>::value), m.Txx);
-      m.Tyy = fma(p2, even(syy, ic<G::sum(SL, l, 1, 1)>::value), m.Tyy);
-      m.Txy = fma(p2, even(sxy, ic<G::sum(SL, l, 0, 1)>::value), m.Txy);
-      m.Txz = fma(p2, even(sxz, ic<G::sum(SL, l, 0, 2)>::value), m.Txz);
-      m.Tyz = fma(p2, even(syz, ic<G::sum(SL, l, 1, 2)>::value), m.Tyz);
+      m.Txx = fma(p2, dbl(sxx), m.Txx);
+      m.Tyy = fma(p2, dbl(syy), m.Tyy);
+      m.Txy = fma(p2, dbl(sxy), m.Txy);
+      m.Txz = fma(p2, dbl(sxz), m.Txz);
+      m.Tyz = fma(p2, dbl(syz), m.Tyz);
     }
   });
   if (!finite) m.N0 = m.T00 = __longlong_as_double(0x7ff8000000000000ll);
