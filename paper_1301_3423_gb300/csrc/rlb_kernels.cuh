@@ -1788,6 +1788,19 @@ __device__ __forceinline__ LevCoef<L, FF> level_coef_ff(FF n, FF T, FF x) {
   return r;
 }
 
+// The same from double coefficients, for cells whose powers of T or n / T leave the range of a float on the
+// way to coefficients that do not (out of line: few cells have such a state).
+template <class L>
+static __device__ __noinline__ LevCoef<L, FF> level_coef_wide(double n, double T, double g) {
+  const LevCoef<L, double> d = level_coef<L, double>(eq_coef<L::ORDER, double>(n, T, g));
+  LevCoef<L, FF> r;
+  static_for<L::NLEV>([&](auto K) {
+    constexpr int l = decltype(K)::value;
+    r.a[l] = ff_from(d.a[l]), r.b[l] = ff_from(d.b[l]), r.c[l] = ff_from(d.c[l]), r.d[l] = ff_from(d.d[l]);
+  });
+  return r;
+}
+
 template <class L, class S>
 __global__ void __launch_bounds__(128) k_init(const double* __restrict__ n, const double* __restrict__ Tf,
                                               const double* __restrict__ u, typename S::T* __restrict__ dst,
@@ -1835,7 +1848,12 @@ __global__ void __launch_bounds__(128) k_init(const double* __restrict__ n, cons
     // beside the float work: 40 % busy); the coefficients, 110 double operations a cell and the bound
     // of this kernel while they were double, are float-float.  128^3 float: 364 us, 876 before; bound
     // by float issue (4640 warp instructions per 32 cells, issue slots 67 %, FMA pipe 63 % used).
-    const LevCoef<L, FF> e = level_coef_ff<L>(ff_from(nn), ff_from(T), ff_from(fma(T, g, -1.0)));
+    // Their intermediate powers go up to T^3 g^3 and down to T / n: in float up to 1e9 and from 1e-9 on,
+    // and with room below for the low parts (1e-25 of 1e-38).
+    const FF nf = ff_from(nn), Tf = ff_from(T), xf = ff_from(fma(T, g, -1.0));
+    LevCoef<L, FF> e;
+    if (Tf.hi > 1e-9f && xf.hi < 1e9f && nf.hi > 1e-25f && nf.hi < 1e25f) e = level_coef_ff<L>(nf, Tf, xf);
+    else e = level_coef_wide<L>(nn, T, g);
     // U / R times 1 .. 6 per axis: t = v.U / R is then a sum of at most three of them
     FF m[3][7];
     const double Ua[3] = {Ux * L::INV_R, Uy * L::INV_R, Uz * L::INV_R};
