@@ -1,4 +1,5 @@
 // C ABI of librlb (declared in include/rlb.h): context management, validation, kernel launches.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -486,19 +487,38 @@ static double* mapped_host(const double* p, size_t count) {
   return static_cast<double*>(a.devicePointer);
 }
 
-// True if array p[0 .. count) is memory of the context's device (both its ends are), so that a kernel
-// may write it; anything else goes through cudaMemcpyAsync, which checks the address.
+// True if array p[0 .. count) lies in one allocation of the context's device, so that a kernel may write
+// it.  Anything else (another device's or managed memory, an array that runs past its allocation or spans
+// two) goes through cudaMemcpyAsync, which checks the whole range itself.
 static bool on_this_device(const rlb_ctx* c, const double* p, size_t count) {
-  const double* const ends[2] = {p, p + (count - 1)};
-  for (const double* q : ends) {
-    cudaPointerAttributes a{};
-    if (cudaPointerGetAttributes(&a, q) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    if (a.type != cudaMemoryTypeDevice || a.device != c->device) return false;
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
   }
-  return (reinterpret_cast<uintptr_t>(p) & 7) == 0;
+  if (a.type != cudaMemoryTypeDevice || a.device != c->device) return false;
+  if ((reinterpret_cast<uintptr_t>(p) & 7) != 0) return false;
+  // the driver call, which libcudart does not wrap; without it every array is copied
+  using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const Range range = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      fn = nullptr;
+    }
+    return reinterpret_cast<Range>(fn);
+  }();
+  if (!range) return false;
+  return in_one_allocation(
+      [](uintptr_t q, uintptr_t* base, size_t* size) {
+        CUdeviceptr b = 0;
+        const bool ok = range(&b, size, (CUdeviceptr)q) == CUDA_SUCCESS;
+        *base = (uintptr_t)b;
+        return ok;
+      },
+      reinterpret_cast<uintptr_t>(p), count * sizeof(double));
 }
 
 extern "C" rlb_status rlb_init(rlb_ctx* c, const double* n, const double* T, const double* u, int on_device) {

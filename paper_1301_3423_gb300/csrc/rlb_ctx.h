@@ -2,11 +2,25 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <cstddef>
+#include <cstdint>
 #include <string>
 
 #include "rlb.h"
 #include "rlb_common.h"
 #include "rlb_launch.h"
+
+namespace rlb {
+// True if [p, p + bytes) lies in the one allocation that holds p, as range(p, &base, &size) reports it (false
+// if p is in none).
+template <class Range>
+bool in_one_allocation(Range range, uintptr_t p, size_t bytes) {
+  uintptr_t base = 0;
+  size_t size = 0;
+  if (!range(p, &base, &size)) return false;
+  return p >= base && p - base <= size && bytes <= size - (p - base);
+}
+}  // namespace rlb
 
 struct rlb_ctx {
   rlb_params prm;
