@@ -211,9 +211,10 @@ rlb_status rlb_autotune(rlb_ctx* ctx, int reps, int* variant, double ms[RLB_MAX_
  * of the row-tile kernel (with two warps per float cell only those whose rows do not fill segment
  * tiles), members that fill a 96-cell row tile better than a 128-cell one through a launch of the
  * 96-cell row-tile kernel with the same warps (variant 19 beside 16), and the other pipelined
- * members through the row-segment kernel of the same block layout.  The others (e.g. 1 x 1 x N
- * tubes) run through the team kernel (float storages; one launch) or, double, the register kernels
- * (see rlb_batch_member_variant).  Members keep
+ * members through the row-segment kernel of the same block layout.  The others run as they would
+ * alone: through the team kernel (1 x 1 x N tubes and boxes up to about 116,000 cells; one launch),
+ * larger ones, and every such double member, through the register kernels (two launches; see
+ * rlb_batch_member_variant).  Members keep
  * their own buffers, parameters, status and step counters; a member's populations after a batched
  * run are bitwise those of the same steps taken alone with the same step-kernel variant.  Members
  * must use the batch's stream.
@@ -256,7 +257,8 @@ rlb_status rlb_batch_set_variant(rlb_batch* b, int variant);
  * variant: the batch's own; the 96-cell row-tile variant for a member that runs in those beside a
  * 128-cell row-tile variant; for a row-tile variant and a member that runs in row segments, the
  * row-segment variant of the same block layout; for a pipelined variant and a member whose rows do
- * not suit the tiles, the fallback (20 float storages, 0 double).  Running that member
+ * not suit the tiles, the fallback (float storages: 20 for a small one, else 3 float and 2 half;
+ * double: 0).  Running that member
  * alone with this variant gives the same populations bitwise.  -1 for an empty slot or NULL. */
 int rlb_batch_member_variant(const rlb_batch* b, int slot);
 

@@ -189,18 +189,11 @@ static bool variant_available(const rlb_ctx* c, int v) {
   return pipe_shape(c, v, nullptr, nullptr, nullptr, nullptr);
 }
 
-// Lattices the team kernel is for: at most this many tiles per resident block (float storages 4, about
-// 116,000 cells; double 1, 14,600).  Measured per step against the register kernels: 1 x 1 x 2613 float
-// 6.7 us against 33, 32^3 float 17 against 25, 64^3 84 against 87, 151 x 93 x 70 512 against 409;
-// 1 x 1 x 800 double 28 us against 104, 96^3 4.7 ms against 2.3 (there the pipe is busy either way and the
-// team's second and third pass through its code cost more).  They also take several steps per launch: a
-// barrier over the grid is about 1 us, the gap between launches 2 to 4.  64 steps in one launch stay below
-// 20 ms.
+// Steps of a small lattice (small_for_team) in one launch of the team kernel: a barrier over the grid is
+// about 1 us, the gap between launches 2 to 4.  64 steps in one launch stay below 20 ms.
 constexpr int kTeamMaxSteps = 64;
 static bool small_for_team(const rlb_ctx* c) {
-  const long long tiles = ((long long)c->cells + kTeamCells - 1) / kTeamCells;
-  const long long room = (long long)c->sms * c->launch->team_resident(c->sp.has_wall);
-  return tiles <= (c->prm.storage == RLB_F64 ? 1 : 4) * room;
+  return small_for_team(c->cells, (int)c->elem, c->sms, c->launch->team_resident(c->sp.has_wall));
 }
 
 // The row-tile variant whose tiles the lattice's rows fill best (at least 3/4 of the lanes), -1 if none.
@@ -249,7 +242,7 @@ static int default_variant(const rlb_ctx* c) {
         pipe_fits(c->sp.nx, lay.tx, (int)c->elem, fill_eighths(lay, (int)c->elem)) && variant_available(c, seg))
       return seg;
   }
-  return small_for_team(c) ? kTeamVariant : (c->prm.storage == RLB_F32 ? 3 : (c->prm.storage == RLB_F16DEV ? 2 : 0));
+  return small_for_team(c) ? kTeamVariant : register_variant(c->prm.storage);
 }
 
 static rlb_status check_launch(rlb_ctx* c, cudaError_t e, const char* what);

@@ -46,8 +46,8 @@ struct rlb_batch {
   int variant = 0;               // step variant: 0..3 register kernels for every member; 4 and up the
                                  // pipelined kernel for the members whose rows suit it (row tiles for
                                  // rows_fit members if the variant has row tiles, row segments for
-                                 // pipe_fits members) and the register fallback (reg_fallback) for the others
-  int walls = 0;                 // some register-kernel member of the uploaded table has bounce-back walls
+                                 // pipe_fits members) and fallback_variant for the others
+  int walls = 0;                 // some team or register-kernel member of the uploaded table has bounce-back walls
   int row_tiles = 0, shell_tiles = 0;  // of the uploaded table: row tiles first, then shell tiles
   int* d_pipe_tm = nullptr;      // member index of every pipelined tile of the uploaded table
   int pipe_tm_capacity = 0;
@@ -114,9 +114,15 @@ extern "C" rlb_status rlb_batch_create(int order, int storage, void* stream, rlb
 
 static int elem_of(int storage) { return storage == RLB_F64 ? 8 : (storage == RLB_F32 ? 4 : 2); }
 
-// The register-kernel variant for members the pipelined kernel cannot take (rows not on 16-byte
-// boundaries): the one a context of that storage runs when no pipelined variant exists for it.
-static int reg_fallback(const rlb_batch* b) { return b->storage == RLB_F64 ? 0 : kTeamVariant; }
+// The variant of a member that a pipelined variant cannot take (rows off 16-byte boundaries, or too few of
+// the tiles' lanes used).  Float storages: what a context of that size runs alone, the team kernel up to
+// about 116,000 cells and the register kernels above; both kinds step in the same run, each by its own
+// launches.  Double storage: the register kernel.
+static int fallback_variant(const rlb_batch* b, const StepParams& p) {
+  const int elem = elem_of(b->storage);
+  if (elem < 8 && small_for_team(p.cells, elem, b->sms, b->launch->team_resident(p.has_wall))) return kTeamVariant;
+  return register_variant(b->storage);
+}
 
 static bool variant_exists(const rlb_batch* b, int v, PipeLayout* lay = nullptr) {
   if (v < 0) return false;
@@ -130,8 +136,8 @@ static bool variant_exists(const rlb_batch* b, int v, PipeLayout* lay = nullptr)
 static int row_tile_fill(int nx, int tx) { return nx <= tx ? (tx / nx) * nx : 0; }
 
 // How a member runs under step variant v: 3 the 96-cell row tiles beside a 128-cell row-tile
-// variant, 2 the variant's row tiles, 1 row segments (pipelined kernel), 0 the register kernels
-// (variant v itself, or reg_fallback for a pipelined v).  A member takes the row tiles whose lanes
+// variant, 2 the variant's row tiles, 1 row segments (pipelined kernel), 0 the register or team kernel
+// (variant v itself, or fallback_variant for a pipelined v).  A member takes the row tiles whose lanes
 // it fills the larger share of (96-cell rows: all of a 96-cell tile against 3/4 of a 128-cell one).
 // Rows that fill segment tiles go to row tiles too, except with two warps per float cell (measured
 // on GB300 at 128^3: one warp per float cell 1.13x faster in row tiles, half storage 1.26x; two
@@ -247,8 +253,8 @@ extern "C" long rlb_batch_steps_left(const rlb_batch* b, int slot) {
 }
 
 // Member table of a run with step variant `variant`: the active members in slot order with their
-// tile ranges (pipelined tiles for the members the pipelined kernel takes, register-kernel row and
-// shell tiles for the others).
+// tile ranges (pipelined tiles for the members the pipelined kernel takes, team tiles or register-kernel
+// row and shell tiles for the others).
 static rlb_status upload_table(rlb_batch* b, long nsteps, int variant, int* nmembers, int* total_tiles) {
   std::vector<BatchMember> t;
   std::vector<int> row_tm, shell_tm, pipe_tm, rtile_tm;
@@ -256,7 +262,6 @@ static rlb_status upload_table(rlb_batch* b, long nsteps, int variant, int* nmem
   b->pipe_walls = 0;
   b->pipe_timeout = nullptr;
   const bool pipe = is_pipe(variant) && variant_exists(b, variant, &b->lay);
-  const bool team = (pipe ? reg_fallback(b) : variant) == kTeamVariant;
   if (!pipe) b->lay = PipeLayout{};
   b->v96 = pipe ? companion96(b, variant, &b->lay96) : -1;
   if (!pipe) b->lay96 = PipeLayout{};
@@ -284,7 +289,7 @@ static rlb_status upload_table(rlb_batch* b, long nsteps, int variant, int* nmem
       continue;
     }
     if (d.p.has_wall) b->walls = 1;
-    if (team) {
+    if ((pipe ? fallback_variant(b, d.p) : variant) == kTeamVariant) {
       d.team_tile_begin = (int)team_tm.size();
       team_tm.resize(team_tm.size() + (d.p.cells + kTeamCells - 1) / kTeamCells, (int)t.size());
       t.push_back(d);
@@ -370,8 +375,8 @@ static rlb_status ensure_counters(rlb_batch* b, long nsteps) {
 
 static int grid_of(rlb_batch* b, int variant) { return b->sms * b->launch->batch_blocks_per_sm(variant); }
 
-// One time step (launch index k) of the uploaded table: the pipelined kernel over its tiles, then
-// the register kernels (row tiles, shell tiles) over the other members' tiles.
+// One time step (launch index k) of the uploaded table: the pipelined kernel over its tiles, then the team
+// kernel and the register kernels (row tiles, shell tiles) over the other members' tiles.
 static rlb_status enqueue_step(rlb_batch* b, int k, int variant, int* counters) {
   cudaError_t e = cudaSuccess;
   // row segments, 128-cell row tiles, 96-cell row tiles
@@ -393,7 +398,7 @@ static rlb_status enqueue_step(rlb_batch* b, int k, int variant, int* counters) 
     if (e != cudaSuccess) return bfail(b, RLB_ECUDA, std::string("batched team step: ") + cudaGetErrorString(e));
   }
   if (b->row_tiles + b->shell_tiles > 0) {
-    const int rv = is_pipe(variant) ? reg_fallback(b) : variant;
+    const int rv = is_pipe(variant) ? register_variant(b->storage) : variant;
     e = b->launch->batch_step(b->d_members, b->d_tile_member, b->row_tiles, b->shell_tiles, k, counters, rv, b->walls,
                               grid_of(b, rv), b->stream);
     b->launches += (b->row_tiles > 0) + (b->shell_tiles > 0);
@@ -554,14 +559,15 @@ extern "C" int rlb_batch_member_variant(const rlb_batch* b, int slot) {
   if (!b || slot < 0 || slot >= (int)b->members.size() || !b->members[slot].ctx) return -1;
   if (!is_pipe(b->variant)) return b->variant;
   PipeLayout lay;
-  if (!variant_exists(b, b->variant, &lay)) return reg_fallback(b);
+  const StepParams& p = b->members[slot].ctx->sp;
+  if (!variant_exists(b, b->variant, &lay)) return fallback_variant(b, p);
   PipeLayout lay96;
   const int v96 = companion96(b, b->variant, &lay96);
-  const int mode = member_mode(b, b->members[slot].ctx->sp, b->variant, lay, lay96);
+  const int mode = member_mode(b, p, b->variant, lay, lay96);
   if (mode == 3) return v96;
   if (mode == 2) return b->variant;
   if (mode == 1) return segment_sibling(b->variant);
-  return reg_fallback(b);
+  return fallback_variant(b, p);
 }
 
 extern "C" long rlb_batch_kernel_launches(const rlb_batch* b) { return b ? b->launches : -1; }

@@ -83,6 +83,19 @@ inline bool rows_fit(int nx, int tx, int elem, int bc_x, int vmax_x) {
   return rows_possible(nx, tx, elem, bc_x, vmax_x) && 4 * (tx / nx) * nx >= 3 * tx;
 }
 
+// The register-kernel variant of a storage (RLB_F64, RLB_F32, RLB_F16DEV) for lattices that suit neither
+// the pipelined kernel nor the team kernel.
+inline int register_variant(int storage) { return storage == 1 ? 3 : (storage == 2 ? 2 : 0); }
+
+// Lattices the team kernel is for: at most this many tiles per resident block (float storages 4, about
+// 116,000 cells; double 1, 14,600).  Measured per step against the register kernels: 1 x 1 x 2613 float
+// 6.7 us against 33, 32^3 float 17 against 25, 64^3 84 against 87, 151 x 93 x 70 512 against 409;
+// 1 x 1 x 800 double 28 us against 104, 96^3 4.7 ms against 2.3 (there the pipe is busy either way and the
+// team's second and third pass through its code cost more).
+inline bool small_for_team(long long cells, int elem, int sms, int resident) {
+  return (cells + kTeamCells - 1) / kTeamCells <= (elem == 8 ? 1LL : 4LL) * sms * resident;
+}
+
 // Tiles of one lattice: row tiles (groups of tx / nx rows) or tx-cell row segments.
 inline long long pipe_tile_count(int nx, int ny, int nz, int tx, int rows) {
   if (rows) {
