@@ -94,7 +94,10 @@ typedef struct {
   void* stream;       /* cudaStream_t to enqueue on; NULL = the default stream */
   int debug_flags;    /* testing only, 0 in normal use.  Bit 0: the pipelined step kernel's producer
                          warps do nothing, so its consumers' bounded waits (2 s) run out and the next
-                         synchronising call reports RLB_ETIMEOUT; the context stays usable. */
+                         synchronising call reports RLB_ETIMEOUT; the context stays usable.  Bit 1:
+                         launches of several steps ask for twice the blocks that fit, so the library
+                         takes one step per launch.  Bit 2: their barrier waits for a block that is
+                         not there, with the same outcome as bit 0. */
   /* Optional quadrature (Sec. II.C, App. A).  When q > 0 these arrays are compared with the
    * quadrature compiled into the library for this order and must match exactly (RLB_EINVAL
    * otherwise); rlb_quadrature() returns the built-in one. */

@@ -193,7 +193,7 @@ static bool variant_available(const rlb_ctx* c, int v) {
 // about 1 us, the gap between launches 2 to 4.  64 steps in one launch stay below 20 ms.
 constexpr int kTeamMaxSteps = 64;
 static bool small_for_team(const rlb_ctx* c) {
-  return small_for_team(c->cells, (int)c->elem, c->sms, c->launch->team_resident(c->sp.has_wall));
+  return small_for_team(c->cells, (int)c->elem, c->team_blocks);
 }
 
 // The row-tile variant whose tiles the lattice's rows fill best (at least 3/4 of the lanes), -1 if none.
@@ -253,8 +253,8 @@ static rlb_status check_launch(rlb_ctx* c, cudaError_t e, const char* what);
 static rlb_status launch_step(rlb_ctx* c, int v) {
   if (v == kTeamVariant)
     return check_launch(c,
-                        c->launch->team_steps(c->buf[c->cur], c->buf[1 - c->cur], c->sp, c->status, 1, c->sms,
-                                              reinterpret_cast<unsigned*>(c->status + kBarrierWord), c->stream),
+                        c->launch->team_steps(c->buf[c->cur], c->buf[1 - c->cur], c->sp, c->status, 1, 0, nullptr,
+                                              c->stream),
                         "team step kernel");
   if (v >= kNumRegVariants) {
     PipeParams pp;
@@ -354,6 +354,7 @@ extern "C" rlb_status rlb_create(const rlb_params* p, rlb_ctx** out) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e == cudaSuccess) {
+    c->team_blocks = c->sms * c->launch->team_resident(c->sp.has_wall);
     const int want = p->step_variant;
     c->variant = (want >= 0 && variant_available(c, want)) ? want : default_variant(c);
     // a variant that was asked for takes one launch per step, as the autotuner times it
@@ -570,13 +571,21 @@ extern "C" rlb_status rlb_step(rlb_ctx* c, long nsteps) {
   while (nsteps > 0) {
     const int k = c->variant == kTeamVariant ? (int)std::min<long>(nsteps, c->team_chunk) : 1;
     rlb_status st = RLB_OK;
-    if (k > 1)
-      st = check_launch(c,
-                        c->launch->team_steps(c->buf[c->cur], c->buf[1 - c->cur], c->sp, c->status, k, c->sms,
-                                              reinterpret_cast<unsigned*>(c->status + kBarrierWord), c->stream),
-                        "team step kernel");
-    else
+    if (k > 1) {
+      const int blocks = c->sp.debug & kDebugTeamGrid ? 2 * c->team_blocks : c->team_blocks;
+      const cudaError_t e = c->launch->team_steps(c->buf[c->cur], c->buf[1 - c->cur], c->sp, c->status, k, blocks,
+                                                  reinterpret_cast<unsigned*>(c->status + kBarrierWord), c->stream);
+      if (e == cudaErrorCooperativeLaunchTooLarge) {
+        // fewer blocks fit now than when the context was made (a device shared by other means): nothing
+        // was launched, and one step per launch needs no block to wait for another
+        cudaGetLastError();
+        c->team_chunk = 1;
+        continue;
+      }
+      st = check_launch(c, e, "team step kernel");
+    } else {
       st = launch_step(c, c->variant);
+    }
     if (st != RLB_OK) return st;
     c->cur = (c->cur + k) & 1;
     c->have_prev = true;

@@ -63,6 +63,7 @@ struct rlb_batch {
   int* d_team_tm = nullptr;      // member index of every team tile
   int team_tm_capacity = 0;
   int team_tiles = 0;
+  int team_resident[2] = {-1, -1};  // blocks per SM of the team kernel without and with walls (-1: not asked)
   int* pipe_timeout = nullptr;   // status word that counts the pipelined kernel's expired waits
   PipeLayout lay{};              // block layout of the current pipelined variant
   int sms = 0, smem_per_sm = 0, smem_optin = 0;
@@ -118,9 +119,9 @@ static int elem_of(int storage) { return storage == RLB_F64 ? 8 : (storage == RL
 // the tiles' lanes used).  Float storages: what a context of that size runs alone, the team kernel up to
 // about 116,000 cells and the register kernels above; both kinds step in the same run, each by its own
 // launches.  Double storage: the register kernel.
-static int fallback_variant(const rlb_batch* b, const StepParams& p) {
+static int fallback_variant(const rlb_batch* b, const rlb_ctx* c) {
   const int elem = elem_of(b->storage);
-  if (elem < 8 && small_for_team(p.cells, elem, b->sms, b->launch->team_resident(p.has_wall))) return kTeamVariant;
+  if (elem < 8 && small_for_team(c->cells, elem, c->team_blocks)) return kTeamVariant;
   return register_variant(b->storage);
 }
 
@@ -289,7 +290,7 @@ static rlb_status upload_table(rlb_batch* b, long nsteps, int variant, int* nmem
       continue;
     }
     if (d.p.has_wall) b->walls = 1;
-    if ((pipe ? fallback_variant(b, d.p) : variant) == kTeamVariant) {
+    if ((pipe ? fallback_variant(b, m.ctx) : variant) == kTeamVariant) {
       d.team_tile_begin = (int)team_tm.size();
       team_tm.resize(team_tm.size() + (d.p.cells + kTeamCells - 1) / kTeamCells, (int)t.size());
       t.push_back(d);
@@ -393,7 +394,10 @@ static rlb_status enqueue_step(rlb_batch* b, int k, int variant, int* counters) 
     if (e != cudaSuccess) return bfail(b, RLB_ECUDA, std::string("batched pipelined step: ") + cudaGetErrorString(e));
   }
   if (b->team_tiles > 0) {
-    e = b->launch->team_batch_step(b->d_members, b->d_team_tm, b->team_tiles, k, b->walls, b->sms, b->stream);
+    int& resident = b->team_resident[b->walls];
+    if (resident < 0) resident = b->launch->team_batch_resident(b->walls);
+    e = b->launch->team_batch_step(b->d_members, b->d_team_tm, b->team_tiles, k, b->walls, b->sms * resident,
+                                   b->stream);
     ++b->launches;
     if (e != cudaSuccess) return bfail(b, RLB_ECUDA, std::string("batched team step: ") + cudaGetErrorString(e));
   }
@@ -559,15 +563,15 @@ extern "C" int rlb_batch_member_variant(const rlb_batch* b, int slot) {
   if (!b || slot < 0 || slot >= (int)b->members.size() || !b->members[slot].ctx) return -1;
   if (!is_pipe(b->variant)) return b->variant;
   PipeLayout lay;
-  const StepParams& p = b->members[slot].ctx->sp;
-  if (!variant_exists(b, b->variant, &lay)) return fallback_variant(b, p);
+  const rlb_ctx* c = b->members[slot].ctx;
+  if (!variant_exists(b, b->variant, &lay)) return fallback_variant(b, c);
   PipeLayout lay96;
   const int v96 = companion96(b, b->variant, &lay96);
-  const int mode = member_mode(b, p, b->variant, lay, lay96);
+  const int mode = member_mode(b, c->sp, b->variant, lay, lay96);
   if (mode == 3) return v96;
   if (mode == 2) return b->variant;
   if (mode == 1) return segment_sibling(b->variant);
-  return fallback_variant(b, p);
+  return fallback_variant(b, c);
 }
 
 extern "C" long rlb_batch_kernel_launches(const rlb_batch* b) { return b ? b->launches : -1; }

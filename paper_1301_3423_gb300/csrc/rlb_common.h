@@ -119,7 +119,11 @@ enum : int {
 constexpr int kBarrierWord = 32, kStatusAlloc = 64;
 
 // StepParams::debug bits (testing only)
-enum : int { kDebugStallProducers = 1 };  // the pipelined step's producers do nothing: every wait runs out
+enum : int {
+  kDebugStallProducers = 1,  // the pipelined step's producers do nothing: every wait runs out
+  kDebugTeamGrid = 2,        // several steps per launch ask for twice the blocks that fit: one step per launch
+  kDebugStallTeam = 4        // their barrier waits for one block more than there are: every wait runs out
+};
 
 // Launch shape of a pipelined step (k_step_pipe, k_step_pipe_batch): tiles are TX-cell segments of
 // the lattice rows, tile t = row * ceil(nx / TX) + seg, or with row tiles groups of TX / nx

@@ -44,6 +44,7 @@ struct rlb_ctx {
   const rlb::Launchers* launch = nullptr;
   int variant = 0;            // step-kernel variant (kNumRegVariants register kernels, then pipelined shapes)
   int team_chunk = 1;         // time steps the team variant takes in one launch
+  int team_blocks = 0;        // blocks of that launch that the device holds at a time
   int device = 0;
   int sms = 0, smem_per_sm = 0, smem_optin = 0;  // device: SMs, shared memory per SM, per block (opt-in)
   // host transfers of rlb_init / rlb_moments run in chunks on a copy stream that overlaps the

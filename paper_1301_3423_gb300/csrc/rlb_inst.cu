@@ -125,7 +125,7 @@ cudaError_t pipe_batch_step(const BatchMember* m, const int* tm, int launch, con
 #define RLB_NAME(o, s) RLB_CAT_(launchers_o, o, _s, s)
 extern const Launchers RLB_NAME(RLB_INST_ORDER, RLB_INST_STORAGE) = {
     step, fields, init, convert_pops, inst::kVariants, batch_step, batch_blocks_per_sm, pipe_step,
-    RLB_TFN(steps), RLB_TFN(resident), RLB_TFN(batch), pipe_batch_step};
+    RLB_TFN(steps), RLB_TFN(resident), RLB_TFN(batch_resident), RLB_TFN(batch), pipe_batch_step};
 
 #if RLB_INST_ORDER == 3 && RLB_INST_STORAGE == 0
 cudaError_t launch_reduce_partials(const double* partial, int nblocks, double* totals, cudaStream_t s) {

@@ -74,10 +74,11 @@ RLB_DECLARE_ROWS(256)
 
 // Team kernels (rlb_inst_team.cu).
 #define RLB_TFN(fn) RLB_CAT7(team_, fn, _o, RLB_INST_ORDER, _s, RLB_INST_STORAGE, )
-cudaError_t RLB_TFN(steps)(void* a, void* b, const StepParams& p, int* status, int nsteps, int sms, unsigned* arrived,
-                           cudaStream_t s);
+cudaError_t RLB_TFN(steps)(void* a, void* b, const StepParams& p, int* status, int nsteps, int blocks,
+                           unsigned* arrived, cudaStream_t s);
 int RLB_TFN(resident)(int walls);
-cudaError_t RLB_TFN(batch)(const BatchMember* m, const int* tm, int ntiles, int launch, int walls, int sms,
+int RLB_TFN(batch_resident)(int walls);
+cudaError_t RLB_TFN(batch)(const BatchMember* m, const int* tm, int ntiles, int launch, int walls, int blocks,
                            cudaStream_t s);
 
 RLB_DECLARE_VARIANT(0)

@@ -34,14 +34,16 @@ struct Launchers {
   cudaError_t (*pipe_step)(const void* src, void* dst, const StepParams& p, const PipeParams& pp, int* status, int tx,
                            int rows, int split, int grid, int threads, int smem, cudaStream_t s);
   // nsteps time steps of the team kernel from buffer a into buffer b and back (one launch; more than
-  // one step is a cooperative launch whose blocks wait for each other, counted in *arrived)
-  cudaError_t (*team_steps)(void* a, void* b, const StepParams& p, int* status, int nsteps, int sms, unsigned* arrived,
-                            cudaStream_t s);
-  // blocks per SM of that launch
+  // one step is a cooperative launch of at most `blocks` blocks, which wait for each other, counted in
+  // *arrived)
+  cudaError_t (*team_steps)(void* a, void* b, const StepParams& p, int* status, int nsteps, int blocks,
+                            unsigned* arrived, cudaStream_t s);
+  // blocks of that launch, and of the batched one, that an SM of the current device holds (0: not known)
   int (*team_resident)(int walls);
+  int (*team_batch_resident)(int walls);
   // one time step (launch index `launch`) of the batch members' team tiles
   cudaError_t (*team_batch_step)(const BatchMember* members, const int* tile_member, int ntiles, int launch, int walls,
-                                 int sms, cudaStream_t s);
+                                 int blocks, cudaStream_t s);
   // one time step of the batched pipelined kernel (launch index `launch`) over the members' tiles;
   // walls != 0 selects the kernel with the bounce-back patch
   cudaError_t (*pipe_batch_step)(const BatchMember* members, const int* tile_member, int launch, const PipeParams& pp,
@@ -87,13 +89,13 @@ inline bool rows_fit(int nx, int tx, int elem, int bc_x, int vmax_x) {
 // the pipelined kernel nor the team kernel.
 inline int register_variant(int storage) { return storage == 1 ? 3 : (storage == 2 ? 2 : 0); }
 
-// Lattices the team kernel is for: at most this many tiles per resident block (float storages 4, about
+// Lattices the team kernel is for: at most this many tiles per block that the device holds (float storages 4, about
 // 116,000 cells; double 1, 14,600).  Measured per step against the register kernels: 1 x 1 x 2613 float
 // 6.7 us against 33, 32^3 float 17 against 25, 64^3 84 against 87, 151 x 93 x 70 512 against 409;
 // 1 x 1 x 800 double 28 us against 104, 96^3 4.7 ms against 2.3 (there the pipe is busy either way and the
 // team's second and third pass through its code cost more).
-inline bool small_for_team(long long cells, int elem, int sms, int resident) {
-  return (cells + kTeamCells - 1) / kTeamCells <= (elem == 8 ? 1LL : 4LL) * sms * resident;
+inline bool small_for_team(long long cells, int elem, int blocks) {
+  return (cells + kTeamCells - 1) / kTeamCells <= (elem == 8 ? 1LL : 4LL) * blocks;
 }
 
 // Tiles of one lattice: row tiles (groups of tx / nx rows) or tx-cell row segments.

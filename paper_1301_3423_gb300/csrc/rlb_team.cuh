@@ -254,13 +254,13 @@ __global__ void __launch_bounds__(kTeamWarps * 32, kTeamBlocks<typename S::A>)
 }
 
 // nsteps time steps in one cooperative launch: block b takes tiles b, b + grid, ...; after each step
-// every block adds 1 to *arrived (0 at launch) and waits until all of the grid have (at most
+// every block adds 1 to *arrived (0 at launch) and waits until all `peers` of the grid have (at most
 // kTeamWaitNs; a wait that runs out is counted and ends the block).  A step reads what other SMs wrote
 // in the one before: the loads go to L2 (__ldcg).
 template <class L, class S, bool WALLS>
 __global__ void __launch_bounds__(kTeamWarps * 32, kTeamBlocks<typename S::A>)
     k_steps_team(typename S::T* a, typename S::T* b, const __grid_constant__ StepParams p, int* status, int ntiles,
-                 int nsteps, unsigned* arrived) {
+                 int nsteps, unsigned* arrived, unsigned peers) {
   __shared__ __align__(16) unsigned char smem[team_smem_bytes<L, S>()];
   __shared__ int gone;
   for (int s = 0; s < nsteps; ++s) {
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(kTeamWarps * 32, kTeamBlocks<typename S::A>)
     if (threadIdx.x == 0) {
       __threadfence();
       atomicAdd(arrived, 1u);
-      const unsigned want = (unsigned)(s + 1) * gridDim.x;
+      const unsigned want = (unsigned)(s + 1) * peers;
       unsigned long long t0 = 0, now;
       gone = 0;
       for (;;) {
