@@ -17,8 +17,9 @@ from paper_1301_3423_gb300 import RLB  # noqa: E402
                                  (1e-10, 1.0), (1e-39, 1e-10), (1.0, 1e-28), (1.0, 1e28)])
 @pytest.mark.parametrize("v", [0.0, 0.5])
 def test_float_initial_state_at_every_scale(order, T, n, v):
-    """32 roundings of 2^-24: three multiply-adds a population, whose terms at the levels that are evaluated
-    in float are up to ten times the value, on coefficients that are rounded once."""
+    """At rest: 32 roundings of 2^-24 of each population, three multiply-adds whose terms at the levels that are
+    evaluated in float are up to ten times the value, on coefficients that are rounded once.  In motion a
+    population may be a small difference of its terms, so only that it is finite."""
     shape = (2, 3, 43)
     u = np.zeros((3,) + shape)
     u[0], u[1], u[2] = 0.6 * v, -0.64 * v, 0.48 * v
@@ -28,5 +29,7 @@ def test_float_initial_state_at_every_scale(order, T, n, v):
             g.init(np.full(shape, n), np.full(shape, T), u)
             f[storage] = g.populations()
     assert np.abs(f["f64"]).max() < 3e38 and np.all(np.isfinite(f["f32"]))
+    if v > 0:
+        return
     scale = np.abs(f["f64"]).max(axis=(1, 2, 3), keepdims=True) + 2.0 ** -126
     assert np.max(np.abs(f["f32"] - f["f64"]) / scale) < 32 * 2.0 ** -24
