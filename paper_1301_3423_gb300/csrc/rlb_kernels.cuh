@@ -567,6 +567,18 @@ struct Landau {
   bool conv;  // the last update moved U by at most tol * U0 (false: stopped at MAXIT)
 };
 
+// a.b = a0 b0 - ax bx - ay by - az bz: the product ax bx rounded, the others as multiply-adds.  Written out,
+// like the products below that something is subtracted from: which of them the compiler contracts depends on
+// the code around, and a cell has to come out the same in every kernel.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+template <class A>
+__device__ __forceinline__ A minkowski(A a0, A ax, A ay, A az, A b0, A bx, A by, A bz) {
+  return fma(-az, bz, fma(-ay, by, fma(a0, b0, -mul_rn(ax, bx))));
+}
+
 // Shifted power iteration from the start vector (U0, Ux, Uy, Uz), at most MAXIT updates; a lane
 // stops once an update moves U by at most tol * U0.
 template <class A, int MAXIT>
@@ -575,16 +587,16 @@ __device__ __forceinline__ Landau<A> landau_from(const Mom<A>& m, A U0, A Ux, A 
   r.ok = false;
   r.conv = false;
   for (int it = 0; it < MAXIT; ++it) {
-    const A V0 = m.T00 * U0 - m.T0x * Ux - m.T0y * Uy - m.T0z * Uz;
-    const A Vx = m.T0x * U0 - m.Txx * Ux - m.Txy * Uy - m.Txz * Uz;
-    const A Vy = m.T0y * U0 - m.Txy * Ux - m.Tyy * Uy - m.Tyz * Uz;
-    const A Vz = m.T0z * U0 - m.Txz * Ux - m.Tyz * Uy - m.Tzz * Uz;
-    const A s = (U0 * V0 - Ux * Vx - Uy * Vy - Uz * Vz) * A(1.0 / 3.0);
+    const A V0 = minkowski(m.T00, m.T0x, m.T0y, m.T0z, U0, Ux, Uy, Uz);
+    const A Vx = minkowski(m.T0x, m.Txx, m.Txy, m.Txz, U0, Ux, Uy, Uz);
+    const A Vy = minkowski(m.T0y, m.Txy, m.Tyy, m.Tyz, U0, Ux, Uy, Uz);
+    const A Vz = minkowski(m.T0z, m.Txz, m.Tyz, m.Tzz, U0, Ux, Uy, Uz);
+    const A s = minkowski(U0, Ux, Uy, Uz, V0, Vx, Vy, Vz) * A(1.0 / 3.0);
     const A W0 = fma(s, U0, V0), Wx = fma(s, Ux, Vx), Wy = fma(s, Uy, Vy), Wz = fma(s, Uz, Vz);
-    const A WW = W0 * W0 - Wx * Wx - Wy * Wy - Wz * Wz;
+    const A WW = minkowski(W0, Wx, Wy, Wz, W0, Wx, Wy, Wz);
     if (!(WW > A(0)) || !(W0 > A(0))) return r;
     const A iw = rsqrt_(WW);
-    const A n0 = W0 * iw, nx = Wx * iw, ny = Wy * iw, nz = Wz * iw;
+    const A n0 = mul_rn(W0, iw), nx = mul_rn(Wx, iw), ny = mul_rn(Wy, iw), nz = mul_rn(Wz, iw);
     const A d = fmax(fmax(fabs(n0 - U0), fabs(nx - Ux)), fmax(fabs(ny - Uy), fabs(nz - Uz)));
     U0 = n0; Ux = nx; Uy = ny; Uz = nz;
     if (d <= tol * U0) {
@@ -592,12 +604,12 @@ __device__ __forceinline__ Landau<A> landau_from(const Mom<A>& m, A U0, A Ux, A 
       break;
     }
   }
-  const A V0 = m.T00 * U0 - m.T0x * Ux - m.T0y * Uy - m.T0z * Uz;
-  const A Vx = m.T0x * U0 - m.Txx * Ux - m.Txy * Uy - m.Txz * Uz;
-  const A Vy = m.T0y * U0 - m.Txy * Ux - m.Tyy * Uy - m.Tyz * Uz;
-  const A Vz = m.T0z * U0 - m.Txz * Ux - m.Tyz * Uy - m.Tzz * Uz;
-  r.eps = U0 * V0 - Ux * Vx - Uy * Vy - Uz * Vz;
-  r.n = U0 * m.N0 - Ux * m.Nx - Uy * m.Ny - Uz * m.Nz;
+  const A V0 = minkowski(m.T00, m.T0x, m.T0y, m.T0z, U0, Ux, Uy, Uz);
+  const A Vx = minkowski(m.T0x, m.Txx, m.Txy, m.Txz, U0, Ux, Uy, Uz);
+  const A Vy = minkowski(m.T0y, m.Txy, m.Tyy, m.Tyz, U0, Ux, Uy, Uz);
+  const A Vz = minkowski(m.T0z, m.Txz, m.Tyz, m.Tzz, U0, Ux, Uy, Uz);
+  r.eps = minkowski(U0, Ux, Uy, Uz, V0, Vx, Vy, Vz);
+  r.n = minkowski(U0, Ux, Uy, Uz, m.N0, m.Nx, m.Ny, m.Nz);
   r.U0 = U0; r.Ux = Ux; r.Uy = Uy; r.Uz = Uz;
   r.ok = (r.eps > A(0)) && (r.n > A(0)) && isfinite(r.eps) && isfinite(r.n);
   return r;
@@ -607,7 +619,7 @@ __device__ __forceinline__ Landau<A> landau_from(const Mom<A>& m, A U0, A Ux, A 
 // place), float at 3e-7 U0.
 template <class A, int MAXIT>
 __device__ __forceinline__ Landau<A> landau(const Mom<A>& m) {
-  const A NN = m.N0 * m.N0 - m.Nx * m.Nx - m.Ny * m.Ny - m.Nz * m.Nz;
+  const A NN = minkowski(m.N0, m.Nx, m.Ny, m.Nz, m.N0, m.Nx, m.Ny, m.Nz);
   if (!(NN > A(0)) || !(m.N0 > A(0))) {
     Landau<A> r;
     r.ok = false;
@@ -631,7 +643,7 @@ __device__ __forceinline__ Landau<A> landau(const Mom<A>& m) {
 template <int MAXIT>
 static __device__ __noinline__ Landau<double> landau_f64(const Mom<double> m) {
   const float N0 = (float)m.N0, Nx = (float)m.Nx, Ny = (float)m.Ny, Nz = (float)m.Nz;
-  const float NN = N0 * N0 - Nx * Nx - Ny * Ny - Nz * Nz;
+  const float NN = minkowski(N0, Nx, Ny, Nz, N0, Nx, Ny, Nz);
   if (N0 > 0.f && 16.f * NN > N0 * N0 && N0 < 1e15f && N0 > 1e-15f) {
     const Mom<float> t = convert<double, float>(m);
     const Landau<float> lf = landau<float, 8>(t);
@@ -640,11 +652,11 @@ static __device__ __noinline__ Landau<double> landau_f64(const Mom<double> m) {
       double U0 = sqrt(fma(Ux, Ux, fma(Uy, Uy, fma(Uz, Uz, 1.0))));
       const float u0 = (float)U0, e1 = lf.eps, k = 0.75f / e1, tiny = 3e-11f * u0;
       for (int it = 0; it < 4; ++it) {
-        const double V0 = m.T00 * U0 - m.T0x * Ux - m.T0y * Uy - m.T0z * Uz;
-        const double Vx = m.T0x * U0 - m.Txx * Ux - m.Txy * Uy - m.Txz * Uz;
-        const double Vy = m.T0y * U0 - m.Txy * Ux - m.Tyy * Uy - m.Tyz * Uz;
-        const double Vz = m.T0z * U0 - m.Txz * Ux - m.Tyz * Uy - m.Tzz * Uz;
-        const double eps = U0 * V0 - Ux * Vx - Uy * Vy - Uz * Vz;
+        const double V0 = minkowski(m.T00, m.T0x, m.T0y, m.T0z, U0, Ux, Uy, Uz);
+        const double Vx = minkowski(m.T0x, m.Txx, m.Txy, m.Txz, U0, Ux, Uy, Uz);
+        const double Vy = minkowski(m.T0y, m.Txy, m.Tyy, m.Tyz, U0, Ux, Uy, Uz);
+        const double Vz = minkowski(m.T0z, m.Txz, m.Tyz, m.Tzz, U0, Ux, Uy, Uz);
+        const double eps = minkowski(U0, Ux, Uy, Uz, V0, Vx, Vy, Vz);
         const float r0 = (float)fma(-eps, U0, V0), rx = (float)fma(-eps, Ux, Vx), ry = (float)fma(-eps, Uy, Vy),
                     rz = (float)fma(-eps, Uz, Vz);
         float d0 = k * r0, dx = k * rx, dy = k * ry, dz = k * rz;
@@ -667,7 +679,7 @@ static __device__ __noinline__ Landau<double> landau_f64(const Mom<double> m) {
           Landau<double> r;
           r.U0 = U0, r.Ux = Ux, r.Uy = Uy, r.Uz = Uz;
           r.eps = eps;  // of the U before the last correction: second order in it
-          r.n = U0 * m.N0 - Ux * m.Nx - Uy * m.Ny - Uz * m.Nz;
+          r.n = minkowski(U0, Ux, Uy, Uz, m.N0, m.Nx, m.Ny, m.Nz);
           r.ok = r.eps > 0.0 && r.n > 0.0 && isfinite(r.eps) && isfinite(r.n);
           r.conv = true;
           return r;
@@ -684,7 +696,7 @@ static __device__ __noinline__ Landau<double> landau_f64(const Mom<double> m) {
 // float, so more digits carry no information, while the double arithmetic still removes the
 // gamma^2 cancellation in U.U = 1.
 static __device__ __noinline__ Landau<double> landau_fp64_out_of_line(const Mom<double> m) {
-  const double NN = m.N0 * m.N0 - m.Nx * m.Nx - m.Ny * m.Ny - m.Nz * m.Nz;
+  const double NN = minkowski(m.N0, m.Nx, m.Ny, m.Nz, m.N0, m.Nx, m.Ny, m.Nz);
   if (!(NN > 0.0) || !(m.N0 > 0.0)) {
     Landau<double> r;
     r.ok = false;
@@ -713,7 +725,7 @@ __device__ __forceinline__ Landau<A> landau_step(const Mom<A>& m, const StepPara
     }
     return r;
   } else {
-    const float NN = m.N0 * m.N0 - m.Nx * m.Nx - m.Ny * m.Ny - m.Nz * m.Nz;
+    const float NN = minkowski(m.N0, m.Nx, m.Ny, m.Nz, m.N0, m.Nx, m.Ny, m.Nz);
     Landau<float> r;
     const bool dbl = p.landau_fp64 || m.N0 * m.N0 > p.gamma_thr2 * NN;
     if (!dbl) {
@@ -755,16 +767,16 @@ template <int ORDER, class A>
 __device__ __forceinline__ EqCoef<ORDER, A> eq_coef(A n, A T, A U0) {
   EqCoef<ORDER, A> c;
   const A x = fma(T, U0, A(-1));
-  const A x2 = x * x, T2 = T * T;
+  const A x2 = mul_rn(x, x), T2 = mul_rn(T, T);
   c.x = x;
   c.T = T;
   if constexpr (ORDER == 3) {
     const A pref = n / (A(12) * T);
     c.pref = pref;
-    c.c00 = A(-6) * pref * (fma(x2, fma(A(8), x, A(4)), fma(A(4), x, A(-2))) + T2 * fma(A(-4), x, A(1)));
-    c.c10 = A(6) * pref * (fma(x2, fma(A(12), x, A(8)), fma(A(5), x, A(-1))) + T2 * fma(A(-6), x, A(1)));
-    c.c01 = A(6) * pref * T * (fma(A(12), x2, A(3)) - A(2) * T2);
-    c.c20 = A(-3) * pref * x * (fma(x, fma(A(6), x, A(3)), A(2)) - A(2) * T2);
+    c.c00 = A(-6) * pref * fma(T2, fma(A(-4), x, A(1)), fma(x2, fma(A(8), x, A(4)), fma(A(4), x, A(-2))));
+    c.c10 = A(6) * pref * fma(T2, fma(A(-6), x, A(1)), fma(x2, fma(A(12), x, A(8)), fma(A(5), x, A(-1))));
+    c.c01 = A(6) * pref * T * fma(A(-2), T2, fma(A(12), x2, A(3)));
+    c.c20 = A(-3) * pref * x * fma(A(-2), T2, fma(x, fma(A(6), x, A(3)), A(2)));
     c.c11 = A(-6) * pref * T * (fma(x, fma(A(6), x, A(1)), A(1)) - T2);
     c.c02 = A(-3) * pref * T2 * fma(A(6), x, A(-1));
   } else {
@@ -794,6 +806,7 @@ struct LevCoef {
 template <class L, class A>
 __device__ __forceinline__ LevCoef<L, A> level_coef(const EqCoef<L::ORDER, A>& q, A shift = A(0)) {
   LevCoef<L, A> r;
+  const A c00 = shift == A(0) ? q.c00 : sub_rn(q.c00, shift);
   static_for<L::NLEV>([&](auto K) {
     constexpr int l = decltype(K)::value;
     constexpr double pd = L::P0[l];
@@ -804,13 +817,13 @@ __device__ __forceinline__ LevCoef<L, A> level_coef(const EqCoef<L::ORDER, A>& q
       r.d[l] = pp3 * (q.T * q.T * q.T);
       r.c[l] = fma(A(3) * ppx, q.T * q.T, p2 * q.c02);
       r.b[l] = fma(A(3) * ppx * q.x, q.T, fma(p2, q.c11, p * q.c01));
-      r.a[l] = fma(ppx * q.x, q.x, fma(p2, q.c20, fma(p, q.c10, q.c00 - shift)));
+      r.a[l] = fma(ppx * q.x, q.x, fma(p2, q.c20, fma(p, q.c10, c00)));
     } else {
       const A pp2 = p2 * q.pref;  // pref p0^2
       r.d[l] = A(0);
       r.c[l] = pp2 * (q.T * q.T);
       r.b[l] = fma(A(2) * pp2 * q.x, q.T, p * q.c01);
-      r.a[l] = fma(pp2 * q.x, q.x, fma(p, q.c10, q.c00 - shift));
+      r.a[l] = fma(pp2 * q.x, q.x, fma(p, q.c10, c00));
     }
   });
   return r;
@@ -1675,7 +1688,7 @@ __global__ void __launch_bounds__(kMomThreads) k_fields(const typename S::T* __r
     // solves, or everywhere with landau_fp64
     const Mom<float> mf = mom_of<float>(m);
     finite = all_finite(mf);
-    const float NN = mf.N0 * mf.N0 - mf.Nx * mf.Nx - mf.Ny * mf.Ny - mf.Nz * mf.Nz;
+    const float NN = minkowski(mf.N0, mf.Nx, mf.Ny, mf.Nz, mf.N0, mf.Nx, mf.Ny, mf.Nz);
     bool dbl = p.landau_fp64 || mf.N0 * mf.N0 > p.gamma_thr2 * NN;
     if (!dbl) {
       const Landau<float> lf = landau<float, 8>(mf);
