@@ -1101,10 +1101,12 @@ __device__ __forceinline__ void relax_cell(Get&& get, Store&& store, const StepP
 // Double arithmetic pulls each population twice (moments, then collision) and has one variant.
 enum StepVariant : int { kRegScalar = 0, kRegPacked = 1, kReg3Scalar = 2, kReg3Packed = 3, kNumVariants = 4 };
 
-template <class S, int VARIANT>
+// The scalar second-order cell asks for 184 registers but fits 168 without spills, so it has 3 blocks either
+// way (160 x 70 x 70 float 120 us a step in two blocks, 106 in three).
+template <class L, class S, int VARIANT>
 struct StepShape {
   static constexpr bool kKeep = std::is_same<typename S::A, float>::value;  // populations in registers
-  static constexpr int kMinBlocks = (VARIANT & 2) ? 3 : 1;
+  static constexpr int kMinBlocks = (VARIANT & 2) || (kKeep && L::ORDER == 2 && !(VARIANT & 1)) ? 3 : 1;
 };
 
 // How a step kernel pulls: the row kernel's warps lie in rows with interior y and z and are told
@@ -1125,7 +1127,7 @@ __device__ __forceinline__ void step_cell(const typename S::T* __restrict__ src,
   using A = typename S::A;
   using ST = typename S::T;
   constexpr bool PACKED = (VARIANT & 1) && std::is_same<A, float>::value;
-  constexpr bool KEEP = StepShape<S, VARIANT>::kKeep;
+  constexpr bool KEEP = StepShape<L, S, VARIANT>::kKeep;
   // Warp-uniform choice: a row warp whose segment is interior pulls with constant offsets; other
   // row warps wrap x only; shell cells resolve wrap / copy-out / bounce-back per population.
   static_assert(PATH == kPathRow || PATH == kPathEdge || PATH == kPathShellTab, "pull path");
@@ -1198,7 +1200,7 @@ __device__ __forceinline__ void row_cell(int w, int lane, const StepParams& p, C
 // interior x range pulls with constant offsets; the others wrap only x.  Whole rows in one kernel
 // keep every sector of a row written by neighbouring warps.
 template <class L, class S, int VARIANT, bool WALLS>
-__global__ void __launch_bounds__(kStepThreads, StepShape<S, VARIANT>::kMinBlocks)
+__global__ void __launch_bounds__(kStepThreads, StepShape<L, S, VARIANT>::kMinBlocks)
     k_step_interior(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
                     const __grid_constant__ StepParams p, int* __restrict__ status) {
   const int w = blockIdx.x * (kStepThreads / 32) + (threadIdx.x >> 5);
@@ -1234,7 +1236,7 @@ __device__ __forceinline__ void shell_row(int r, const StepParams& p, int& y, in
 // blockIdx alone, a value the compiler knows to be the same for the whole warp; as many blocks
 // per SM as the four-warp kernels have warps.
 template <class L, class S, int VARIANT, bool WALLS>
-__global__ void __launch_bounds__(32, 4 * StepShape<S, VARIANT>::kMinBlocks)
+__global__ void __launch_bounds__(32, 4 * StepShape<L, S, VARIANT>::kMinBlocks)
     k_step_shell_rows(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
                       const __grid_constant__ StepParams p, int* __restrict__ status) {
   const int w = blockIdx.x;
@@ -1276,7 +1278,7 @@ __device__ __forceinline__ Cell shell_cell(int s, const StepParams& p) {
 }
 
 template <class L, class S, bool GENERAL, int VARIANT, bool WALLS>
-__global__ void __launch_bounds__(kStepThreads, StepShape<S, VARIANT>::kMinBlocks)
+__global__ void __launch_bounds__(kStepThreads, StepShape<L, S, VARIANT>::kMinBlocks)
     k_step_shell(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
                  const __grid_constant__ StepParams p, int* __restrict__ status) {
   const int s = blockIdx.x * kStepThreads + threadIdx.x;
@@ -1298,7 +1300,7 @@ __global__ void __launch_bounds__(kStepThreads, StepShape<S, VARIANT>::kMinBlock
 // are skipped.
 // ---------------------------------------------------------------------------------------------
 template <class L, class S, int VARIANT, bool WALLS, bool ROWS>
-__global__ void __launch_bounds__(kStepThreads, StepShape<S, VARIANT>::kMinBlocks)
+__global__ void __launch_bounds__(kStepThreads, StepShape<L, S, VARIANT>::kMinBlocks)
     k_step_batch(const BatchMember* __restrict__ members, const int* __restrict__ tile_member, int tile_begin,
                  int tile_end, int launch_index, int* __restrict__ counter) {
   using ST = typename S::T;
