@@ -59,9 +59,9 @@ constexpr int kTeamBlocks = sizeof(A) == 8 ? 3 : 6;
 constexpr int kPipeMaxStages = 16;
 constexpr int kPipeMaxConsumerWarps = 16;
 constexpr int kPipeMaxProducerWarps = 12;
-// Consumers + producers, the launch bound of k_step_pipe: 20 warps of 96 registers for float and half
-// storage, 16 of 128 for double (whose cells need more).
-constexpr int pipe_max_warps(int elem) { return elem == 8 ? 16 : 20; }
+// Consumers + producers, the launch bound of k_step_pipe: 20 warps of 96 registers for float and half storage,
+// 16 of 128 for double (whose cells need more) and for float cells in two warps (whose shapes have no more).
+constexpr int pipe_max_warps(int elem, bool split) { return elem == 8 || (elem == 4 && split) ? 16 : 20; }
 constexpr int kPipeChunks = 4;  // chunks of populations per stage, each with its own barriers
 constexpr int kPipeHeaderBytes = 1536;  // mbarriers (2 x 16 x 4 x 8 B) and the per-population velocity table
 constexpr int kPipeXchgBytesPerPair = 2 * 2 * 13 * 32 * 4;  // partial moments a consumer warp pair exchanges

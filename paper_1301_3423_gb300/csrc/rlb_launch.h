@@ -126,9 +126,9 @@ inline bool pipe_layout(int v, int q, int elem, int smem_per_sm, int smem_optin,
   const bool split = elem == 4 && cf.split;  // float storage: two consumer warps per cell
   const int wpt = cf.tx / 32 * (split ? 2 : 1);
   const int groups = cf.cons_warps / wpt;
-  // The producers that the kernel's warps leave room for: twelve consumer warps leave double storage, whose
-  // cells need 128 registers a thread, four of the eight that float and half storage have.
-  const int room = pipe_max_warps(elem) - cf.cons_warps;
+  // The producers that the kernel's warps leave room for: twelve consumer warps leave four in a block of
+  // 128 registers a thread.
+  const int room = pipe_max_warps(elem, split) - cf.cons_warps;
   const int producers = cf.producers < room ? cf.producers : room;
   if (groups < 1 || cf.cons_warps % wpt != 0 || producers < 1 || producers > q) return false;
   if (producers > kPipeMaxProducerWarps || cf.cons_warps > kPipeMaxConsumerWarps) return false;

@@ -53,8 +53,8 @@
 
 namespace rlb {
 
-template <class S>
-constexpr int kPipeMaxThreads = sizeof(typename S::T) == 8 ? 16 * 32 : 20 * 32;  // pipe_max_warps
+template <class S, bool ONEWARP>
+constexpr int kPipeMaxThreads = 32 * pipe_max_warps(sizeof(typename S::T), !ONEWARP);
 constexpr unsigned long long kPipeWaitNs = 2000000000ull;  // 2 s
 
 // Geometry of one staged row for storage S and tile width TX.
@@ -230,9 +230,11 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
   constexpr int kStageElems = L::Q * BX;
   constexpr bool DEV = std::is_same<S, StoreF16Dev>::value;
   static_assert(TX % 32 == 0 && TX >= 32, "tile width");
-  // Row segments with one warp per float cell release their stage chunk by chunk while they collide;
-  // the others have one chunk, the stage.
-  constexpr bool EARLY = PACKED && !SPLIT && !ROWS;
+  // Row segments with one warp per float cell release their stage chunk by chunk while they collide; the others
+  // have one chunk, the stage.  So have third-order half segments, whose chunks of 32 short copies gain less
+  // than the barriers cost (640 x 35 x 36 139 us a step against 142, 1024 x 27 x 28 147 against 149; second order
+  // 77 against 74 and 97 against 89).
+  constexpr bool EARLY = PACKED && !SPLIT && !ROWS && (!DEV || L::ORDER == 2);
   constexpr int NCH = EARLY ? kPipeChunks : 1, CH = ChunkSize<L, NCH>::value;
 
   extern __shared__ __align__(128) unsigned char smem[];
@@ -404,10 +406,6 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[s * NCH + c]);
     };
-    auto wait_all = [&] {
-#pragma unroll
-      for (int c = 0; c < NCH; ++c) wait_chunk(c);
-    };
     auto release_all = [&] {
       __syncwarp();
       if (lane < NCH) mbar_arrive(&empty[s * NCH + lane]);
@@ -417,6 +415,13 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
       if (!__any_sync(0xffffffffu, late)) return false;
       if (lane == 0) atomicAdd(tiles.timeout_word(), 1);
       return true;
+    };
+    // the chunks after the first, which every tile waits for first of all; true if a wait ran out
+    auto rest_late = [&]() -> bool {
+      if constexpr (NCH == 1) return false;
+#pragma unroll
+      for (int c = 1; c < NCH; ++c) wait_chunk(c);
+      return gave_up();
     };
     // a batch works out the tile's cells and stage offsets (from the member's parameters in
     // memory) before the wait for the stage, so that their loads overlap it; a single lattice, whose
@@ -483,8 +488,7 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
     // last part of a tile of 96-cell rows, a ragged row end): release the stage and leave the issue
     // slots to the other warps (both warps of a float pair skip together)
     if (!tr.active || !__any_sync(0xffffffffu, valid)) {
-      wait_all();
-      if (gave_up()) return;
+      if (rest_late()) return;
       release_all();
       continue;
     }
@@ -502,10 +506,7 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
                         (p.bc[2] == kBounceBack && (cl.z < L::VMAX_Z || cl.z >= p.nz - L::VMAX_Z));
       patch = patch || (ROWS ? __any_sync(0xffffffffu, near) : near);
     }
-    if (patch || !EARLY) {
-      wait_all();
-      if (gave_up()) return;
-    }
+    if (patch && rest_late()) return;
     if (patch) {
       static_for<L::Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
@@ -683,7 +684,7 @@ struct BatchTiles {
 
 // One time step of one lattice.
 template <class L, class S, int TX, bool WALLS, bool ROWS, bool ONEWARP>
-__global__ void __launch_bounds__(kPipeMaxThreads<S>, 1)
+__global__ void __launch_bounds__(kPipeMaxThreads<S, ONEWARP>, 1)
     k_step_pipe(const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
                 const __grid_constant__ StepParams p, const __grid_constant__ PipeParams pp,
                 int* __restrict__ status) {
@@ -695,7 +696,7 @@ __global__ void __launch_bounds__(kPipeMaxThreads<S>, 1)
 // members' tiles.  A member's result is bitwise that of k_step_pipe on it alone.  Waits that run
 // out are counted in *timeout (the first member's status words).
 template <class L, class S, int TX, bool WALLS, bool ROWS, bool ONEWARP>
-__global__ void __launch_bounds__(kPipeMaxThreads<S>, 1)
+__global__ void __launch_bounds__(kPipeMaxThreads<S, ONEWARP>, 1)
     k_step_pipe_batch(const BatchMember* __restrict__ members, const int* __restrict__ tile_member, int launch,
                       const __grid_constant__ PipeParams pp, int* __restrict__ timeout) {
   using T = typename S::T;

@@ -31,10 +31,10 @@ def layout(tmp_path_factory):
                    'extern "C" int layout(int v, int q, int elem, int* out) {\n'
                    "  rlb::PipeLayout l{};\n"
                    "  if (!rlb::pipe_layout(v, q, elem, %d, %d, &l)) return 0;\n"
-                   "  const int r[] = {l.tx, l.rows, l.nstage, l.groups, l.producers, l.threads, l.smem};\n"
-                   "  for (int k = 0; k < 7; ++k) out[k] = r[k];\n"
+                   "  const int r[] = {l.tx, l.rows, l.nstage, l.groups, l.producers, l.threads, l.smem, l.split};\n"
+                   "  for (int k = 0; k < 8; ++k) out[k] = r[k];\n"
                    "  return 1;\n}\n"
-                   'extern "C" int max_warps(int elem) { return rlb::pipe_max_warps(elem); }\n'
+                   'extern "C" int max_warps(int elem, int split) { return rlb::pipe_max_warps(elem, split); }\n'
                    % (SMEM_PER_SM, SMEM_PER_BLOCK))
     cuda = os.path.dirname(os.path.dirname(builder._nvcc()))
     subprocess.check_call([shutil.which("g++") or "g++", "-std=c++17", "-shared", "-fPIC", "-I", builder.CSRC, "-I",
@@ -42,11 +42,11 @@ def layout(tmp_path_factory):
     lib = ctypes.CDLL(str(d / "layout.so"))
 
     def ask(v, order, storage):
-        out = (ctypes.c_int * 7)()
+        out = (ctypes.c_int * 8)()
         if not lib.layout(v, Q[order], ELEM[storage], out):
             return None
-        return dict(zip(("tx", "rows", "nstage", "groups", "producers", "threads", "smem"), out))
-    ask.max_warps = lambda storage: lib.max_warps(ELEM[storage])
+        return dict(zip(("tx", "rows", "nstage", "groups", "producers", "threads", "smem", "split"), out))
+    ask.max_warps = lambda storage, lay: lib.max_warps(ELEM[storage], lay["split"])
     return ask
 
 
@@ -59,7 +59,7 @@ def test_shapes_exist(layout, order, storage):
             got[v] = lay
     assert set(got) == SHAPES[order, storage]
     for lay in got.values():
-        assert lay["threads"] <= 32 * layout.max_warps(storage)
+        assert lay["threads"] <= 32 * layout.max_warps(storage, lay)
         assert lay["nstage"] >= 2 and lay["nstage"] % lay["groups"] == 0 and lay["smem"] <= SMEM_PER_BLOCK
         assert 1 <= lay["producers"] <= lay["threads"] // 32 - 1
 
