@@ -196,30 +196,53 @@ static bool small_for_team(const rlb_ctx* c) {
   return small_for_team(c->cells, (int)c->elem, c->team_blocks);
 }
 
-// The row-tile variant whose tiles the lattice's rows fill best (at least 3/4 of the lanes), -1 if none.
-// Equal fills go to the first in an order measured on GB300: float 128-cell tiles (64^3 57 us a step
-// against 62 in 192-cell tiles, 128^3 351 against 440), then 192 (48^3 29 us against 32 in 96-cell
-// tiles, 96^3 170 against 171), half storage, whose copies are half as long, 192 and 256 (64^3 48 us
-// against 54 in 128-cell tiles, 128^3 315 against 335, 192^3 1.09 ms against 1.39 on the register kernel).
+// The row-tile variant that steps the lattice fastest: the share of the tiles' lanes that the rows use (at least
+// 3/4) times the rate of a full tile, in per cent of the storage's best.  -1 if none fits.  The rates are those
+// of 0.8 M cells with rows of 24 to 256 cells at the third and the second order: float 128-cell tiles 5.7 and 11.8
+// updates a ns at full lanes, 192 5.6 and 12.6, 256 (second order only) 10.4, 160 4.7 and 10.7, 96 5.0 and 9.5;
+// half 256 6.2 and 13.3, 192 5.8 and 11.9 (64-cell rows, which fill both, 6.2 and 6.4), 128 5.8 and 10.4,
+// 160 5.0 and 9.9, 96 4.8 and 9.2.  Equal products go to the first.  (40-cell rows: float in 128-cell tiles
+// 161 us a step, in 160-cell tiles, which they fill, 181; half in 256-cell tiles 140 against 184.)
 // Tiles fewer than the SMs would leave some idle: then the narrowest.
 static int best_row_tiles(const rlb_ctx* c) {
-  static const int order_f32[] = {16, 22, 19, 21, 23}, order_f16[] = {22, 23, 21, 12, 19}, narrow[] = {19, 12, 16, 21, 22, 23};
-  const bool f32 = c->prm.storage == RLB_F32;
-  for (int pass = 0; pass < 2; ++pass) {
-    const int* order = pass ? narrow : (f32 ? order_f32 : order_f16);
-    int best = -1, cells = 0, width = 1;  // of the best so far: cells per tile, tile width
-    for (int k = 0; k < (pass ? 6 : 5); ++k) {
-      if (order[k] == (f32 ? 12 : 16)) continue;  // the slower of the two 128-cell shapes
-      PipeLayout lay;
-      if (!pipe_layout(order[k], c->q, (int)c->elem, c->smem_per_sm, c->smem_optin, &lay)) continue;
-      if (!rows_fit(c->sp.nx, lay.tx, (int)c->elem, c->sp.bc[0], vmax_x(c)) || !variant_available(c, order[k])) continue;
-      if (!pass && pipe_tile_count(c->sp.nx, c->sp.ny, c->sp.nz, lay.tx, 1) < c->sms) continue;
-      const int used = lay.tx / c->sp.nx * c->sp.nx;
-      if (best < 0 || used * width > cells * lay.tx) best = order[k], cells = used, width = lay.tx;
-    }
-    if (best >= 0) return best;
+  struct Tiles {
+    int variant, rate[2];  // third order, second order
+  };
+  static const Tiles f32[] = {{16, {100, 94}}, {22, {100, 100}}, {23, {0, 83}}, {21, {84, 85}}, {19, {85, 76}}};
+  static const Tiles f16[] = {{22, {100, 90}}, {23, {100, 100}}, {12, {88, 78}}, {21, {84, 75}}, {19, {74, 69}}};
+  static const int narrow_f32[] = {19, 16, 21, 22, 23}, narrow_f16[] = {19, 12, 21, 22, 23};
+  const bool is_f32 = c->prm.storage == RLB_F32;
+  auto tile_width = [&](int v) -> int {  // 0 if the lattice does not suit the variant
+    PipeLayout lay;
+    if (!pipe_layout(v, c->q, (int)c->elem, c->smem_per_sm, c->smem_optin, &lay)) return 0;
+    if (!rows_fit(c->sp.nx, lay.tx, (int)c->elem, c->sp.bc[0], vmax_x(c)) || !variant_available(c, v)) return 0;
+    return lay.tx;
+  };
+  int best = -1;
+  double most = 0.0;
+  for (const Tiles& t : is_f32 ? f32 : f16) {
+    const int w = tile_width(t.variant);
+    if (w == 0 || pipe_tile_count(c->sp.nx, c->sp.ny, c->sp.nz, w, 1) < c->sms) continue;
+    const double speed = (double)t.rate[c->prm.order == 2] * (w / c->sp.nx * c->sp.nx) / w;
+    if (speed > most) best = t.variant, most = speed;
   }
+  if (best >= 0) return best;
+  for (int v : is_f32 ? narrow_f32 : narrow_f16)
+    if (tile_width(v) > 0) return v;
   return -1;
+}
+
+// Whether more than 1 in 20 rows of the lattice lie within the stencil's reach of a y or z wall.  The pipelined
+// kernel patches such rows in shared memory population by population, a chain of loads that the register
+// kernels' shell rows do not have.  96^3 with walls on y (one row in 8, second order 16) takes it 479 us a step
+// (float; half 472, second order 185 and 198) against 280 (284, 122 and 117) there; 128 x 256 x 26 (one row in 21,
+// second order 43) 286 (236, 111, 99) against 296 (293, 130, 107).
+static bool many_rows_at_walls(const rlb_ctx* c) {
+  const int vy = c->prm.order == 3 ? Quad3::VMAX_Y : Quad2::VMAX_Y, vz = c->prm.order == 3 ? Quad3::VMAX_Z : Quad2::VMAX_Z;
+  const long long ny = c->sp.ny, nz = c->sp.nz;
+  const long long fy = c->sp.bc[1] == kBounceBack ? std::max(ny - 2 * vy, 0LL) : ny;
+  const long long fz = c->sp.bc[2] == kBounceBack ? std::max(nz - 2 * vz, 0LL) : nz;
+  return 20 * (ny * nz - fy * fz) > ny * nz;
 }
 
 // The variant rlb_step uses unless asked otherwise.  Double storage, whose step is bound by the
@@ -228,25 +251,26 @@ static int best_row_tiles(const rlb_ctx* c) {
 // kernels; narrower segments measured slower than those), then the register kernels (small lattices:
 // the team kernel).
 static int default_variant(const rlb_ctx* c) {
-  if (c->prm.storage != RLB_F64) {
+  if (c->prm.storage != RLB_F64 && !many_rows_at_walls(c)) {
     const int rows = best_row_tiles(c);
     if (rows >= 0) return rows;
     const int seg = 15;
     PipeLayout lay;
-    // An x that is not periodic is patched in shared memory population by population in the first and
-    // last segment of each row, a chain of loads that the register kernels do not have: a job of such
-    // rows ran at 0.6 ns a cell update here, 0.33 to 0.35 on the register kernels (151 x 93 x 70).  So
-    // only where those two segments are less than half of a row.
+    // An x that is not periodic is patched like the rows at walls, in the first and last segment of each row:
+    // 640-cell open rows take 1154 us for 0.8 M cells (float; half 1383) against 222 on the register kernels,
+    // 1024-cell ones 634 against 222 and 150 without patches, so that some 60 segments would hide the two.
+    // Rows that use 3/4 of the lanes suit segments, at the second order of half storage 7/8 (320 cells, 5/6
+    // used: half 189 us against 207 on the register kernels, second order 103 against 91).
     if (pipe_layout(seg, c->q, (int)c->elem, c->smem_per_sm, c->smem_optin, &lay) &&
-        (c->sp.bc[0] == kPeriodic || c->sp.nx > 4 * lay.tx) &&
-        pipe_fits(c->sp.nx, lay.tx, (int)c->elem, fill_eighths(lay, (int)c->elem)) && variant_available(c, seg))
+        (c->sp.bc[0] == kPeriodic || c->sp.nx > 64 * lay.tx) &&
+        pipe_fits(c->sp.nx, lay.tx, (int)c->elem, c->prm.storage == RLB_F16DEV && c->prm.order == 2 ? 7 : 6) &&
+        variant_available(c, seg))
       return seg;
   }
   return small_for_team(c) ? kTeamVariant : register_variant(c->prm.storage);
 }
 
 static rlb_status check_launch(rlb_ctx* c, cudaError_t e, const char* what);
-
 
 // One time step of the whole lattice with step-kernel variant v: the register kernels (two
 // launches: interior rows, then the shell) or the pipelined kernel (one launch).
