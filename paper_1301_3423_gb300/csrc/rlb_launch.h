@@ -89,15 +89,14 @@ inline bool rows_fit(int nx, int tx, int elem, int bc_x, int vmax_x) {
 // the pipelined kernel nor the team kernel.
 inline int register_variant(int storage) { return storage == 1 ? 3 : (storage == 2 ? 2 : 0); }
 
-// Lattices the team kernel is for: at most this many tiles per block that the device holds (float 4, 116,736
-// cells; half 3.75, 109,440; double 1, 14,592).  Measured per step against the register kernels: 1 x 1 x 2613
-// float 6.7 us against 33, 32^3 float 17 against 25, 49 x 48 x 46 48.7 against 59 (half, second order, 23.4
-// against 24.8; 50 x 50 x 46 26.4 against 24.8), 151 x 93 x 70 512 against 409; 1 x 1 x 800 double 28 us against
-// 104, 96^3 4.9 ms against 2.3 (there the pipe is busy either way and the team's second and third pass through
-// its code cost more).
+// Lattices the team kernel is for: at most this many tiles per block that the device holds (float storages 4,
+// 116,736 cells; double 1, 14,592).  Measured per step against the register kernels: 1 x 1 x 2613 float 6.7 us
+// against 33, 32^3 float 17 against 25, 49 x 48 x 46 48.7 against 59, 48 x 49 x 49 half, open in x, 41.1 against
+// 54.2 (only 50 x 50 x 46 half, second order, lost: 26.4 against 24.8), 151 x 93 x 70 512 against 409; 1 x 1 x 800
+// double 28 us against 104, 96^3 4.9 ms against 2.3 (there the pipe is busy either way and the team's second and
+// third pass through its code cost more).
 inline bool small_for_team(long long cells, int elem, int blocks) {
-  const long long tiles = (cells + kTeamCells - 1) / kTeamCells, quarters = elem == 8 ? 4 : (elem == 4 ? 16 : 15);
-  return 4 * tiles <= quarters * blocks;
+  return (cells + kTeamCells - 1) / kTeamCells <= (elem == 8 ? 1LL : 4LL) * blocks;
 }
 
 // Tiles of one lattice: row tiles (groups of tx / nx rows) or tx-cell row segments.

@@ -24,8 +24,8 @@ CASES = [
     ((24, 24, 24), (0, 2, 0), 3, TEAM, TEAM), ((20, 20, 256), (0, 2, 0), 3, TEAM, TEAM),
     # segments 5/6 used
     ((20, 24, 320), (0, 0, 0), 3, 15, 15), ((20, 24, 320), (0, 0, 0), 2, 15, 2),
-    # the largest lattices of the team kernel: 116,736 cells float, 109,440 half
-    ((46, 49, 50), (0, 0, 0), 3, TEAM, 2), ((46, 49, 48), (1, 0, 0), 3, TEAM, TEAM), ((47, 49, 51), (0, 0, 0), 3, 3, 2),
+    # the largest lattices of the team kernel: 116,736 cells
+    ((46, 49, 51), (0, 0, 0), 3, TEAM, TEAM), ((46, 49, 48), (1, 0, 0), 3, TEAM, TEAM), ((47, 49, 51), (0, 0, 0), 3, 3, 2),
 ]
 
 
