@@ -1633,9 +1633,9 @@ static __device__ __noinline__ Landau<double> landau_readout_fp64(const Mom<doub
 // ---------------------------------------------------------------------------------------------
 // fields and conserved densities of one time level.  Double storage: double moments and Landau solve.
 // Float storages: float moments (moments_pd), the step's Landau policy, and one update of a float
-// frame in float-float (frame_update).  128^3 float: 357 us, 0.49 of the copy bandwidth, bound by
-// instruction issue; 767 us with the update in double and every coordinate of every pull wrapped by
-// itself.  Double: 96^3 876 us against 2563 (integer sums, corrected frame).
+// frame in float-float (frame_update).  128^3 float: 357 us, 0.49 of the copy bandwidth, bound by the
+// latency of the pulls (issue slots 44 %, 7 of 12 stalled warps on loads); 767 us with the update in
+// double and every coordinate of every pull wrapped by itself.  Double: 96^3 876 us against 2563 (integer sums, corrected frame).
 //   PULL = true : the pre-collision populations pulled from the previous state
 //   PULL = false: the stored populations of each cell
 // out.f[k][cell], k = n, eps, U0, U1, U2, U3; partial[block][5] = block sums of
@@ -1862,7 +1862,7 @@ __global__ void __launch_bounds__(128) k_init(const double* __restrict__ n, cons
     // inputs are normalised in double (some 40 operations a cell, which the 1/64-rate pipe does
     // beside the float work: 40 % busy); the coefficients, 110 double operations a cell and the bound
     // of this kernel while they were double, are float-float.  128^3 float: 364 us, 876 before; bound
-    // by float issue (4640 warp instructions per 32 cells, issue slots 67 %, FMA pipe 63 % used).
+    // by float issue (4660 warp instructions per 32 cells, issue slots 65 %, FMA pipe 62 % used).
     // Their intermediate powers go up to T^3 g^3 and down to T / n: in float up to 1e9 and from 1e-9 on,
     // and with room below for the low parts (1e-25 of 1e-38).
     const FF nf = ff_from(nn), Tf = ff_from(T), xf = ff_from(fma(T, g, -1.0));

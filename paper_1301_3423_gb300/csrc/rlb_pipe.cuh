@@ -36,8 +36,8 @@
 // tile.  NSTAGE is a multiple of the group count, so each stage is read by one group, and every
 // producer and that group take the stage's uses in order: when either waits for use u of a stage,
 // use u - 1 is complete and use u + 1 cannot be, and the parity of u names the right phase.
-// A stage is one chunk of populations, or four (row segments, one warp per float cell), with a barrier
-// pair each: full[s][c] completes when the chunk's producers have arrived for the stage's tile and
+// A stage is one chunk of populations, or four (row segments of float storage with one warp per cell and of
+// second-order half storage), with a barrier pair each: full[s][c] completes when the chunk's producers have arrived for the stage's tile and
 // their copies have landed, empty[s][c] when every consumer warp of that tile has read the chunk for
 // the last time.  Moments and collision go through the chunks in order, so the next tile's first chunk
 // is on its way while the last is still being collided, and its moments start before its last chunk
