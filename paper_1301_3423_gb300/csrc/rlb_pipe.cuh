@@ -269,6 +269,11 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
     const int pw = warp - cons_warps;
     const int P = pp.producers;
     if (tiles.debug() & kDebugStallProducers) return;  // testing: nothing arrives, every wait runs out
+    // this producer's chunks: c0, c0 + cstep, ...; its populations of a chunk: first, first + share, ...
+    const int c0 = pw % NCH, cstep = P < NCH ? P : NCH;
+    const int share = chunk_producers<NCH>(c0, P), first = P < NCH ? 0 : pw / NCH;
+    const int mine_whole = max(0, (CH - first + share - 1) / share);
+    const int mine_last = max(0, (L::Q - (NCH - 1) * CH - first + share - 1) / share);
     int k = 0;
     bool ok = true;
     for (; ok; ++k) {
@@ -301,12 +306,9 @@ __device__ __forceinline__ void pipe_body(const PipeParams& pp, const Tiles& til
         }
         bulk_g2s(d, src + from, (uint32_t)(n * sizeof(T)), bar);
       };
-      for (int c = pw % NCH; c < NCH; c += P < NCH ? P : NCH) {
+      for (int c = c0; c < NCH; c += cstep) {
         uint64_t* const bar = &full[s * NCH + c];
-        const int share = chunk_producers<NCH>(c, P);  // producers of this chunk; this one's number is first
-        const int first = P < NCH ? 0 : pw / NCH;
-        const int end = min((c + 1) * CH, L::Q);
-        const int mine = max(0, (end - c * CH - first + share - 1) / share);
+        const int mine = c == NCH - 1 ? mine_last : mine_whole;
         if (k >= pp.nstage && !mbar_wait(&empty[s * NCH + c], (uint32_t)((k / pp.nstage) - 1) & 1u)) ok = false;
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
